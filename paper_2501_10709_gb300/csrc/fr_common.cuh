@@ -354,6 +354,10 @@ bool tc_rollout_supported(const fr_env *env, const fr_ensemble *e);
 // writes them (its count restarts with every episode, as the kernel's).
 cudaError_t launch_metrics_replay(const EnvView &v, const int64_t *vlog, int T, double *metrics,
                                   cudaStream_t s, const int32_t *t0 = nullptr);
+// its form without auto-reset (fr_metrics.cu): every env's logged steps are a
+// prefix of the log, which ends with its episode
+cudaError_t launch_episode_replay(const EnvView &v, const int64_t *vlog, int T, double *metrics, cudaStream_t s,
+                                  const int32_t *t0);
 // fused stock rollout with resident weights (fr_fused2.cu)
 bool f2_supported(const fr_env *env, const fr_ensemble *e);
 int f2_rollout(fr_env *env, const fr_ensemble *e, int T, const fr_traj *traj, double *metrics,

@@ -180,18 +180,22 @@ __device__ __forceinline__ void acc_push(double &mu, double &m2, double &mdd,
     vlast = v1;
 }
 
-// {cumulative return, Sharpe = (mu - r_f) / sd * sqrt(A), max drawdown}
+// Sharpe = (mu - r_f) / sd * sqrt(A), r_f = 0; 0 with fewer than two periods
+// or zero variance.
+__device__ __forceinline__ double sharpe_of(double mu, double m2, int n, double ann)
+{
+    if (n < 2 || m2 == 0.0) return 0.0;
+    const double sd = __dsqrt_rn(__ddiv_rn(m2, (double)(n - 1)));
+    return __dmul_rn(__ddiv_rn(__dsub_rn(mu, 0.0), sd), __dsqrt_rn(ann));
+}
+
+// {cumulative return, Sharpe, max drawdown}
 __device__ __forceinline__ void acc_final(double mu, double m2, double mdd,
                                           int64_t vlast, int64_t v0, int n,
                                           double ann, double *out)
 {
     out[0] = __dsub_rn(__ddiv_rn((double)vlast, (double)v0), 1.0);
-    double sh = 0.0;
-    if (n >= 2 && m2 != 0.0) {
-        const double sd = __dsqrt_rn(__ddiv_rn(m2, (double)(n - 1)));
-        sh = __dmul_rn(__ddiv_rn(__dsub_rn(mu, 0.0), sd), __dsqrt_rn(ann));
-    }
-    out[1] = sh;
+    out[1] = sharpe_of(mu, m2, n, ann);
     out[2] = mdd;
 }
 
