@@ -114,6 +114,7 @@ static int use_device(const fr_ctx *ctx)
 cudaError_t forward_plain(const fr_ensemble *e, const float *obs, int ld, int n, float *y,
                           float *scratch, cudaStream_t s)
 {
+    if (mlp_f32_ok(e)) return launch_mlp_f32(e, obs, ld, n, y, s);
     int wmax = 0;
     for (int l = 1; l < e->L; ++l) wmax = std::max(wmax, e->dims[l]);
     const float *in = obs;
@@ -201,7 +202,7 @@ int forward_any(const fr_ensemble *e, const float *obs, int ld, int n, float *y,
         return rc;
     }
     void *scratch = nullptr;
-    const uint64_t sb = plain_scratch_bytes(e, n);
+    const uint64_t sb = mlp_f32_ok(e) ? 0 : plain_scratch_bytes(e, n);
     if (sb) FR_CUDA(cudaMallocAsync(&scratch, sb, s));
     cudaError_t err = forward_plain(e, obs, ld, n, y, (float *)scratch, s);
     if (scratch) cudaFreeAsync(scratch, s);
@@ -1091,7 +1092,7 @@ static int plain_rollout(fr_env *env, const fr_ensemble *e, int32_t T, const fr_
     const bool tiled_ok = !(env->tune_set && !env->tune_tiled);
     const uint64_t tiles_b =
         (e->precision == FR_PREC_FP32 || !tiled_ok) ? 0 : ((tc_tiled_scratch_bytes(e, N) + 255) & ~255ull);
-    const uint64_t need = obs_b + act_b + y_b + tiles_b + plain_scratch_bytes(e, N);
+    const uint64_t need = obs_b + act_b + y_b + tiles_b + (mlp_f32_ok(e) ? 0 : plain_scratch_bytes(e, N));
     if (env->scratch_bytes < need) {
         FR_CUDA(cudaStreamSynchronize(s));
         dev_free(env->ctx, env->scratch, env->scratch_bytes);

@@ -321,7 +321,13 @@ cudaError_t launch_q_targets(const float *Yon, const float *Ytg, int64_t y_strid
 cudaError_t launch_combine_vote(const float *Y, int64_t y_stride, int ldy, int M, int n, int nact,
                                 uint32_t dueling, uint8_t *out, cudaStream_t s);
 
-// Bytes of scratch the plain forward needs for n rows (two hidden buffers).
+// The whole fp32 network in one launch (fr_plain.cu), for the layer widths
+// mlp_f32_ok accepts; the same results as launch_dense_f32 layer by layer.
+bool mlp_f32_ok(const fr_ensemble *e);
+cudaError_t launch_mlp_f32(const fr_ensemble *e, const float *obs, int ld, int n, float *y, cudaStream_t s);
+
+// Bytes of scratch the layer-by-layer forward needs for n rows (two hidden
+// buffers).
 inline uint64_t plain_scratch_bytes(const fr_ensemble *e, int n)
 {
     int w = 0;

@@ -75,6 +75,220 @@ __global__ void __launch_bounds__(NT) k_dense_f32(const float *__restrict__ X, i
     }
 }
 
+// The whole fp32 network of one agent for a tile of BM rows in one block.
+// k_dense_f32 above runs 4 x 4 outputs per thread from scalar shared-memory
+// reads (8 reads per 16 FMAs: 18 TFLOP/s of the 80 the FP32 pipes give) in one
+// launch per layer, with every hidden activation through HBM.  Here:
+//  * the hidden activations stay in shared memory, k-major as the next layer
+//    reads them; a layer's outputs are all in registers when its last k is
+//    done, so one buffer serves every layer;
+//  * a thread holds TM x TN outputs (8 x 8 at 64 rows x 256 columns) and reads
+//    16-byte vectors: a warp is 4 row groups x 8 column groups, so each read is
+//    one wavefront, 4 of them per 64 FMAs;
+//  * the FMAs run two columns per instruction (fma.rn.f32x2);
+//  * weights come from global memory (L2) through registers into a
+//    double-buffered k-major tile, the next one's loads under the current
+//    one's FMAs.
+// Every output is the same chain of FMAs over k as in k_dense_f32: the same
+// bits.  3 x 301-256-256-30, whole call: 8,192 rows 415 -> 211 us (35
+// TFLOP/s), 256 rows 130 -> 53 us, one row 99 -> 53 us.
+constexpr int ML_THREADS = 256;
+constexpr int ML_MAX_K = 304;                 // widest layer input
+constexpr uint32_t ML_STAGE = 8704;           // bytes of a weight tile (2,048 floats, rows padded by 4)
+
+struct MlpArgs {
+    const float *X;
+    int ldx, n;
+    const float *params;
+    int64_t P;
+    int64_t w_off[MAX_LAYERS], b_off[MAX_LAYERS];
+    int dims[MAX_LAYERS + 1];
+    int L, out_act, kmax;
+    float *Y;                                 // [M][n][dims[L]]
+};
+
+__device__ __forceinline__ uint64_t pack2f(float lo, float hi)
+{
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+
+__device__ __forceinline__ void unpack2f(uint64_t v, float &lo, float &hi)
+{
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+
+// d = a * b + d on both halves, each rounded once
+__device__ __forceinline__ void fma2(uint64_t &d, uint64_t a, uint64_t b)
+{
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
+}
+
+// One layer.  NPAD columns (32, 64, 128 or 256 >= fout), weight tiles of BK
+// rows.  As [fin][BM + 4] holds the layer's input and receives its output
+// unless it is the last layer.
+template <int BM, int NPAD>
+__device__ __forceinline__ void mlp_layer(const MlpArgs &a, int l, const float *__restrict__ W,
+                                          const float *__restrict__ B, float *As, float *Ws, int row0, int agent)
+{
+    constexpr int BK = NPAD == 32 ? 32 : 2048 / NPAD;
+    constexpr int TN = NPAD >= 128 ? 8 : 4;
+    constexpr int CW = NPAD / (8 * TN);                   // warps side by side
+    constexpr int RW = 8 / CW;
+    constexpr int TM = BM / (4 * RW) > 0 ? BM / (4 * RW) : 1;
+    constexpr int SA = BM + 4, SW = NPAD + 4;
+    constexpr int QUADS = BK * NPAD / 4 / ML_THREADS;     // 4-column groups of a tile per thread
+    static_assert((uint32_t)(BK * SW * 4) <= ML_STAGE && QUADS >= 1, "weight tile");
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int fin = a.dims[l], fout = a.dims[l + 1];
+    const bool last = l == a.L - 1;
+    const int r0 = (warp / CW) * 4 * TM + (lane >> 3) * TM;            // rows r0 .. r0 + TM - 1
+    const int c0 = (warp % CW) * 8 * TN + (lane & 7) * 4;              // columns c0 .. + 3 (and + 32 ..)
+    const bool active = r0 < BM;
+
+    float stage[QUADS][4];
+    auto load = [&](int k0) {
+#pragma unroll
+        for (int q = 0; q < QUADS; ++q) {
+            const int i = threadIdx.x + q * ML_THREADS, k = k0 + i % BK, c = 4 * (i / BK);
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                stage[q][u] = (k < fin && c + u < fout) ? __ldg(W + (int64_t)(c + u) * fin + k) : 0.0f;
+        }
+    };
+    auto store = [&](int b) {
+#pragma unroll
+        for (int q = 0; q < QUADS; ++q) {
+            const int i = threadIdx.x + q * ML_THREADS;
+            *(float4 *)(Ws + b * (ML_STAGE / 4) + (i % BK) * SW + 4 * (i / BK)) =
+                make_float4(stage[q][0], stage[q][1], stage[q][2], stage[q][3]);
+        }
+    };
+
+    uint64_t acc[TM][TN / 2];
+#pragma unroll
+    for (int i = 0; i < TM; ++i)
+#pragma unroll
+        for (int j = 0; j < TN / 2; ++j) acc[i][j] = 0ull;
+    auto step = [&](const float *ap, const float *wp) {
+        float x[TM];
+        if constexpr (TM >= 4) {
+#pragma unroll
+            for (int i = 0; i < TM; i += 4) *(float4 *)(x + i) = *(const float4 *)(ap + i);
+        } else if constexpr (TM == 2) {
+            *(float2 *)x = *(const float2 *)ap;
+        } else {
+            x[0] = ap[0];
+        }
+        ulonglong2 w[TN / 4];
+#pragma unroll
+        for (int j = 0; j < TN / 4; ++j) w[j] = *(const ulonglong2 *)(wp + 32 * j);
+#pragma unroll
+        for (int i = 0; i < TM; ++i) {
+            const uint64_t xx = pack2f(x[i], x[i]);
+#pragma unroll
+            for (int j = 0; j < TN / 4; ++j) {
+                fma2(acc[i][2 * j], xx, w[j].x);
+                fma2(acc[i][2 * j + 1], xx, w[j].y);
+            }
+        }
+    };
+
+    load(0);
+    store(0);
+    __syncthreads();                                      // the tile, and the layer's input
+    int b = 0;
+    for (int k0 = 0; k0 < fin; k0 += BK, b ^= 1) {
+        const bool more = k0 + BK < fin;
+        if (more) load(k0 + BK);
+        const float *ap = As + k0 * SA + r0, *wp = Ws + b * (ML_STAGE / 4) + c0;
+        const int kn = min(BK, fin - k0);
+        if (active) {
+            if (kn == BK) {
+#pragma unroll
+                for (int k = 0; k < BK; ++k) step(ap + k * SA, wp + k * SW);
+            } else {
+#pragma unroll 1
+                for (int k = 0; k < kn; ++k) step(ap + k * SA, wp + k * SW);
+            }
+        }
+        if (more) store(b ^ 1);
+        __syncthreads();                                  // next tile stored, this one (and at the end As) read
+    }
+
+    if (!active) return;
+#pragma unroll
+    for (int j = 0; j < TN; ++j) {
+        const int c = c0 + (j & 3) + (j >> 2) * 32;
+        const float bias = c < fout ? __ldg(B + c) : 0.0f;
+        float y[TM];
+#pragma unroll
+        for (int i = 0; i < TM; ++i) {
+            float lo, hi;
+            unpack2f(acc[i][j / 2], lo, hi);
+            y[i] = (j & 1 ? hi : lo) + bias;
+        }
+        if (last) {
+#pragma unroll
+            for (int i = 0; i < TM; ++i) {
+                const int r = row0 + r0 + i;
+                if (r < a.n && c < fout)
+                    a.Y[((int64_t)agent * a.n + r) * fout + c] = a.out_act ? tanhf(y[i]) : y[i];
+            }
+        } else if (c < fout) {
+            float *h = As + c * SA + r0;
+#pragma unroll
+            for (int i = 0; i < TM; ++i) y[i] = fmaxf(y[i], 0.0f);
+            if constexpr (TM >= 4) {
+#pragma unroll
+                for (int i = 0; i < TM; i += 4) *(float4 *)(h + i) = *(const float4 *)(y + i);
+            } else if constexpr (TM == 2) {
+                *(float2 *)h = *(const float2 *)y;
+            } else {
+                h[0] = y[0];
+            }
+        }
+    }
+}
+
+template <int BM>
+__global__ void __launch_bounds__(ML_THREADS, 2) k_mlp_f32(const __grid_constant__ MlpArgs a)
+{
+    extern __shared__ float4 ml_smem[];
+    constexpr int SA = BM + 4;
+    float *As = (float *)ml_smem;
+    float *Ws = As + a.kmax * SA;
+    const int agent = blockIdx.y;
+    const int row0 = blockIdx.x * BM;
+    const float *P = a.params + (int64_t)agent * a.P;
+    // the tile's input rows, k-major: four rows per thread, consecutive lanes
+    // consecutive k, one 16-byte store each (conflict-free: rows of 4 (BM + 4)
+    // bytes shift by 16 bytes per k)
+    const int fin = a.dims[0];
+    for (int i = threadIdx.x; i < fin * (BM / 4); i += ML_THREADS) {
+        const int g = i / fin, k = i - g * fin, r = row0 + 4 * g;
+        float v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) v[u] = r + u < a.n ? __ldg(a.X + (int64_t)(r + u) * a.ldx + k) : 0.0f;
+        *(float4 *)(As + k * SA + 4 * g) = make_float4(v[0], v[1], v[2], v[3]);
+    }
+    for (int l = 0; l < a.L; ++l) {
+        const float *W = P + a.w_off[l], *B = P + a.b_off[l];
+        const int N = a.dims[l + 1];
+        if (N > 128)
+            mlp_layer<BM, 256>(a, l, W, B, As, Ws, row0, agent);
+        else if (N > 64)
+            mlp_layer<BM, 128>(a, l, W, B, As, Ws, row0, agent);
+        else if (N > 32)
+            mlp_layer<BM, 64>(a, l, W, B, As, Ws, row0, agent);
+        else
+            mlp_layer<BM, 32>(a, l, W, B, As, Ws, row0, agent);
+    }
+}
+
+uint32_t mlp_smem(int bm, int kmax) { return (uint32_t)(kmax * (bm + 4) * 4) + 2u * ML_STAGE; }
+
 // a = a_0 + sum_{j>=1} w_j (a_j - a_0), rounded at every operation
 __global__ void k_combine_mean(const float *__restrict__ Y, int64_t y_stride, int ldy,
                                const float *__restrict__ w, int M, int n, int K,
@@ -138,6 +352,60 @@ __global__ void k_q_targets(const float *__restrict__ Yon, const float *__restri
 }
 
 }  // namespace
+
+// Networks k_mlp_f32 takes: every input up to 304 wide, every output up to 256.
+bool mlp_f32_ok(const fr_ensemble *e)
+{
+    for (int l = 0; l < e->L; ++l)
+        if (e->dims[l] > ML_MAX_K || e->dims[l + 1] > 256) return false;
+    return true;
+}
+
+cudaError_t launch_mlp_f32(const fr_ensemble *e, const float *obs, int ld, int n, float *y, cudaStream_t s)
+{
+    MlpArgs a = {};
+    a.X = obs;
+    a.ldx = ld;
+    a.n = n;
+    a.params = e->params;
+    a.P = e->P;
+    a.L = e->L;
+    a.out_act = e->out_act;
+    a.Y = y;
+    for (int l = 0; l <= e->L; ++l) a.dims[l] = e->dims[l];
+    for (int l = 0; l < e->L; ++l) {
+        a.w_off[l] = e->w_off[l];
+        a.b_off[l] = e->b_off[l];
+        a.kmax = e->dims[l] > a.kmax ? e->dims[l] : a.kmax;
+    }
+    // Rows per block: an SM's time is its blocks x (rows + a fixed part), so
+    // small batches take short tiles that reach every SM, large ones tall
+    // tiles that read each weight less often (measured, 3 x 301-256-256-30:
+    // 16 rows 53 us up to 810 rows, 64 rows 211 us at 8,192).
+    const int sms = e->ctx->sm_count > 0 ? e->ctx->sm_count : 1;
+    int bm = 64;
+    int64_t best = -1;
+    for (int c : {64, 32, 16}) {
+        const int64_t cost = (int64_t)ceil_div((int64_t)ceil_div(n, c) * e->M, sms) * (c + 12);
+        if (best < 0 || cost < best) {
+            best = cost;
+            bm = c;
+        }
+    }
+    const dim3 grid(ceil_div(n, bm), e->M);
+    const uint32_t smem = mlp_smem(bm, a.kmax);
+    const void *f = bm == 64 ? (const void *)k_mlp_f32<64> : bm == 32 ? (const void *)k_mlp_f32<32>
+                                                                   : (const void *)k_mlp_f32<16>;
+    const cudaError_t err = set_max_smem_once(f, e->ctx->device);
+    if (err != cudaSuccess) return err;
+    if (bm == 64)
+        k_mlp_f32<64><<<grid, ML_THREADS, smem, s>>>(a);
+    else if (bm == 32)
+        k_mlp_f32<32><<<grid, ML_THREADS, smem, s>>>(a);
+    else
+        k_mlp_f32<16><<<grid, ML_THREADS, smem, s>>>(a);
+    return cudaGetLastError();
+}
 
 cudaError_t launch_heads(const float *Y, int64_t y_stride, int ldy, int M, int n, int nact, uint32_t dueling,
                          float *q, cudaStream_t s)
