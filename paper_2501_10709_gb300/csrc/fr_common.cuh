@@ -217,6 +217,24 @@ inline unsigned ceil_div(long long a, long long b) { return (unsigned)((a + b - 
 // no such call and can be captured into a CUDA graph).  fr_api.cu.
 cudaError_t set_max_smem_once(const void *func, int device);
 
+// Launch `kernel` so that its blocks may be placed while the stream's previous
+// kernel still runs; it calls ptx::grid_wait_previous() before it touches
+// anything the previous one wrote or still reads.
+template <class... P, class... A>
+inline cudaError_t launch_after(void (*kernel)(P...), unsigned grid, unsigned block, cudaStream_t s, A... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid, 1, 1);
+    cfg.blockDim = dim3(block, 1, 1);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 // ------------------------------------------------------- kernel launchers
 // env kernels (fr_env_kernels.cu)
 cudaError_t launch_env_reset(const EnvView &v, cudaStream_t s);
@@ -351,6 +369,17 @@ int tc_get_act_scales(const fr_ensemble *e, float *scales);
 uint64_t tc_tiled_scratch_bytes(const fr_ensemble *e, int n);
 int tc_forward_tiled(const fr_ensemble *e, const float *obs, int ld, int n, float *y, void *scratch,
                      cudaStream_t s);
+// Narrow networks with every agent resident in one CTA (fr_narrow.cu): the
+// same results as tc_forward and the fused crypto rollout.
+bool nw_ok(const fr_ensemble *e);
+int nw_forward(const fr_ensemble *e, const float *obs, int ld, int n, float *y, cudaStream_t s);
+// two hidden layers up to 256 wide, weights resident in CTA pairs (fr_wide.cu)
+bool wd_ok(const fr_ensemble *e);
+int wd_forward(const fr_ensemble *e, const float *obs, int ld, int n, float *y, cudaStream_t s);
+// Fewer 128-row tiles than SMs.  Hidden NaNs become 0 (max(x, 0)) in such
+// batches and stay NaN in larger ones.
+inline int tc_small_batch(const fr_ensemble *e, int n) { return (int)ceil_div(n, 128) < e->ctx->sm_count; }
+int nw_rollout(fr_env *env, const fr_ensemble *e, int T, const fr_traj *traj, int64_t *vlog, cudaStream_t s);
 // Whether the fused persistent rollout supports this env / ensemble pair.
 bool tc_rollout_supported(const fr_env *env, const fr_ensemble *e);
 // FP64 episode accumulators from a rollout's value log (fr_fused.cu)

@@ -1005,7 +1005,8 @@ int tc_rollout(fr_env *env, const fr_ensemble *e, int T, const fr_traj *traj, do
     FR_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, env->ctx->device));
     int stages = pick_stages(v.task, p, optin, env->ctx->device, &resident, &ring_bytes);
     FR_CHECK(stages > 0, FR_EINVAL, "fused rollout: plan does not fit in shared memory");
-    if (env->tune_set && env->tune_stages >= 2 && env->tune_stages < stages) {
+    const bool ring = env->tune_set && env->tune_stages >= 2 && env->tune_stages < stages;
+    if (ring) {
         // an autotuned ring: fewer stages, the weights streamed
         stages = env->tune_stages;
         resident = 0;
@@ -1025,6 +1026,14 @@ int tc_rollout(fr_env *env, const fr_ensemble *e, int T, const fr_traj *traj, do
         int rc = dev_alloc(env->ctx, &env->scratch, need);
         if (rc) return rc;
         env->scratch_bytes = need;
+    }
+    if (v.task == FR_TASK_CRYPTO && nw_ok(e) && !ring) {
+        FR_CUDA(env_time_mark(env, 0, s));
+        const int rc = nw_rollout(env, e, T, traj, (int64_t *)env->scratch, s);
+        if (rc) return rc;
+        FR_CUDA(env_time_mark(env, 1, s));
+        FR_CUDA(launch_metrics_replay(v, (const int64_t *)env->scratch, T, metrics, s));
+        return FR_OK;
     }
     FusedArgs a;
     memset(&a, 0, sizeof(a));

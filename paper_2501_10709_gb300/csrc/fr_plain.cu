@@ -3,6 +3,7 @@
 // separate combine launch.  It is the comparison path for the fused BF16
 // rollout and the fp32 reference the tensor-core kernels are held to.
 #include "fr_common.cuh"
+#include "fr_ptx.cuh"
 
 namespace fr {
 
@@ -290,10 +291,11 @@ __global__ void __launch_bounds__(ML_THREADS, 2) k_mlp_f32(const __grid_constant
 uint32_t mlp_smem(int bm, int kmax) { return (uint32_t)(kmax * (bm + 4) * 4) + 2u * ML_STAGE; }
 
 // a = a_0 + sum_{j>=1} w_j (a_j - a_0), rounded at every operation
-__global__ void k_combine_mean(const float *__restrict__ Y, int64_t y_stride, int ldy,
+__global__ void k_combine_mean(const float *Y, int64_t y_stride, int ldy,
                                const float *__restrict__ w, int M, int n, int K,
                                float *__restrict__ out, int ldo)
 {
+    ptx::grid_wait_previous();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= (int64_t)n * K) return;
     const int64_t r = i / K, k = i % K;
@@ -306,9 +308,10 @@ __global__ void k_combine_mean(const float *__restrict__ Y, int64_t y_stride, in
 
 // per-agent argmax (lowest index on ties), then the action with the strictly
 // largest count, else hold (1)
-__global__ void k_combine_vote(const float *__restrict__ Y, int64_t y_stride, int ldy, int M,
+__global__ void k_combine_vote(const float *Y, int64_t y_stride, int ldy, int M,
                                int n, int nact, uint32_t dueling, uint8_t *__restrict__ out)
 {
+    ptx::grid_wait_previous();
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= n) return;
     int cnt[3] = {0, 0, 0};
@@ -326,9 +329,10 @@ __global__ void k_combine_vote(const float *__restrict__ Y, int64_t y_stride, in
 }
 
 // Q-values after each agent's head: q[j][r][a], a < nact.
-__global__ void k_heads(const float *__restrict__ Y, int64_t y_stride, int ldy, int M, int n, int nact,
+__global__ void k_heads(const float *Y, int64_t y_stride, int ldy, int M, int n, int nact,
                         uint32_t dueling, float *__restrict__ q)
 {
+    ptx::grid_wait_previous();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= (int64_t)M * n) return;
     const int j = (int)(i / n), r = (int)(i % n);
@@ -337,10 +341,11 @@ __global__ void k_heads(const float *__restrict__ Y, int64_t y_stride, int ldy, 
 }
 
 // DQN / Double DQN learning targets y[j][r] = r + (done ? 0 : gamma Q_target(s', a*)).
-__global__ void k_q_targets(const float *__restrict__ Yon, const float *__restrict__ Ytg, int64_t y_stride, int ldy,
+__global__ void k_q_targets(const float *Yon, const float *Ytg, int64_t y_stride, int ldy,
                             int M, int n, int nact, uint32_t dueling, const float *__restrict__ rew,
                             const uint8_t *__restrict__ done, float gamma, int double_q, float *__restrict__ y)
 {
+    ptx::grid_wait_previous();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= (int64_t)M * n) return;
     const int j = (int)(i / n), r = (int)(i % n);
@@ -410,17 +415,15 @@ cudaError_t launch_mlp_f32(const fr_ensemble *e, const float *obs, int ld, int n
 cudaError_t launch_heads(const float *Y, int64_t y_stride, int ldy, int M, int n, int nact, uint32_t dueling,
                          float *q, cudaStream_t s)
 {
-    k_heads<<<ceil_div((int64_t)M * n, 256), 256, 0, s>>>(Y, y_stride, ldy, M, n, nact, dueling, q);
-    return cudaGetLastError();
+    return launch_after(k_heads, ceil_div((int64_t)M * n, 256), 256u, s, Y, y_stride, ldy, M, n, nact, dueling, q);
 }
 
 cudaError_t launch_q_targets(const float *Yon, const float *Ytg, int64_t y_stride, int ldy, int M, int n, int nact,
                              uint32_t dueling, const float *rew, const uint8_t *done, float gamma, int double_q,
                              float *y, cudaStream_t s)
 {
-    k_q_targets<<<ceil_div((int64_t)M * n, 256), 256, 0, s>>>(Yon, Ytg, y_stride, ldy, M, n, nact, dueling, rew,
-                                                               done, gamma, double_q, y);
-    return cudaGetLastError();
+    return launch_after(k_q_targets, ceil_div((int64_t)M * n, 256), 256u, s, Yon, Ytg, y_stride, ldy, M, n, nact, dueling,
+                        rew, done, gamma, double_q, y);
 }
 
 cudaError_t launch_dense_f32(const float *X, int64_t x_stride, int ldx, const float *P,
@@ -467,15 +470,13 @@ cudaError_t launch_combine_mean(const float *Y, int64_t y_stride, int ldy, const
                                 int n, int K, float *out, int ldo, cudaStream_t s)
 {
     const int64_t tot = (int64_t)n * K;
-    k_combine_mean<<<ceil_div(tot, 256), 256, 0, s>>>(Y, y_stride, ldy, w, M, n, K, out, ldo);
-    return cudaGetLastError();
+    return launch_after(k_combine_mean, ceil_div(tot, 256), 256u, s, Y, y_stride, ldy, w, M, n, K, out, ldo);
 }
 
 cudaError_t launch_combine_vote(const float *Y, int64_t y_stride, int ldy, int M, int n, int nact,
                                 uint32_t dueling, uint8_t *out, cudaStream_t s)
 {
-    k_combine_vote<<<ceil_div(n, 256), 256, 0, s>>>(Y, y_stride, ldy, M, n, nact, dueling, out);
-    return cudaGetLastError();
+    return launch_after(k_combine_vote, ceil_div(n, 256), 256u, s, Y, y_stride, ldy, M, n, nact, dueling, out);
 }
 
 }  // namespace fr

@@ -569,6 +569,8 @@ int tc_forward(const fr_ensemble *e, const float *obs, int ld, int n, float *y, 
     FR_CHECK(t, FR_EINVAL, "tensor-core image missing");
     FR_CHECK(t->plan.esz != 1 || t->scaled, FR_ENOTREADY,
              "FP8 ensemble needs activation scales (ensemble_set_act_scales or ensemble_calibrate_sync)");
+    if (nw_ok(e)) return nw_forward(e, obs, ld, n, y, s);
+    if (wd_ok(e)) return wd_forward(e, obs, ld, n, y, s);
     dim3 grid(ceil_div(n, 128), e->M);
     k_tc_forward<<<grid, TC_THREADS, tc_smem_bytes(t->plan), s>>>(t->plan, t->img, t->bias, t->dq, t->inv_sx,
                                                                   obs, ld, n, y, t->err);

@@ -127,5 +127,79 @@ __device__ __forceinline__ void split_pack8(const float *v, uint32_t *hi, uint32
     }
 }
 
+// warp_wait_all after one poll: a phase that is already complete costs no
+// look at the abort flag.
+__device__ __forceinline__ bool quick_wait(uint64_t *bar, uint32_t parity, volatile int *abort, unsigned *err,
+                                        unsigned code)
+{
+    if (__all_sync(0xffffffffu, ptx::mbar_try_wait(bar, parity))) return true;
+    return ptx::warp_wait_all(bar, parity, false, abort, err, code, TC_WAIT_NS);
+}
+
+// a + b and both halves at once
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b)
+{
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
+// Accumulators a, b plus the bias pair, ReLU, rounded to two 16-bit operands.
+// A NaN stays NaN, or (NAN0) becomes 0 as max(x, 0) makes it.
+template <bool NAN0>
+__device__ __forceinline__ uint32_t relu2(uint32_t a, uint32_t b, uint64_t bias2, bool f16)
+{
+    uint64_t v;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "r"(a), "r"(b));
+    v = add2(v, bias2);
+    float lo, hi;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+    if (NAN0) {
+        lo = fmaxf(lo, 0.0f);
+        hi = fmaxf(hi, 0.0f);
+    }
+    return f16 ? ptx::relu_f16x2_sat(lo, hi) : ptx::relu_bf16x2(lo, hi);
+}
+
+// One unit's accumulators (this thread's lane, n columns of tensor memory from
+// acc: the rows of a transposed layer) + bias, ReLU, as operand words: eight
+// rows at a time, put(g, w) with w[4] the words of rows 8 g .. 8 g + 7.
+// loaded() runs once the last accumulator is in registers.
+template <bool NAN0, class Put, class Loaded>
+__device__ __forceinline__ void unit_rows(uint32_t acc, float bias, int n, bool f16, Put put, Loaded loaded)
+{
+    using namespace ptx;
+    uint64_t b2;
+    asm("mov.b64 %0, {%1, %1};" : "=l"(b2) : "f"(bias));
+    int c0 = 0;
+    for (; c0 + 32 <= n; c0 += 32) {
+        uint32_t v[32];
+        __syncwarp();
+        tmem_ld32(acc + (uint32_t)c0, v);
+        tmem_ld_wait();
+        if (c0 + 32 == n) loaded();
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+            uint32_t w[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) w[i] = relu2<NAN0>(v[8 * g + 2 * i], v[8 * g + 2 * i + 1], b2, f16);
+            put(c0 / 8 + g, w);
+        }
+    }
+    if (c0 < n) {
+        uint32_t v[16];
+        __syncwarp();
+        tmem_ld16(acc + (uint32_t)c0, v);
+        tmem_ld_wait();
+        loaded();
+#pragma unroll
+        for (int g = 0; g < 2; ++g) {
+            uint32_t w[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) w[i] = relu2<NAN0>(v[8 * g + 2 * i], v[8 * g + 2 * i + 1], b2, f16);
+            put(c0 / 8 + g, w);
+        }
+    }
+}
 
 }  // namespace fr

@@ -1,0 +1,522 @@
+// fr_wide.cu -- the stock ensemble's networks (two hidden layers up to 256
+// wide, inputs up to 304, up to 32 outputs; BF16 or FP16) as a batch forward
+// with resident weights, for every batch size.
+//
+// One agent's 303 KB of weights do not fit one SM's operand memory twice
+// over, so a pair of CTAs (a cluster of two) shares an agent: CTA c computes
+// units 128 c .. 128 c + 127 of both hidden layers for the pair's tile of up
+// to 64 rows.  Its halves of the first two layers sit in tensor memory (152 +
+// 128 columns at 301-256-256-30) for as long as the CTA lives, where the MMA
+// reads them at full rate (an A operand in shared memory takes 1.2 to 1.5
+// times as long), and the small output layer in shared memory.  The layers run
+// transposed, D[unit][row] = W[unit][k] X[k][row]: M = 128 units, N = the
+// tile's rows, so that a batch of eight rows pays for sixteen and not for 128,
+// a thread's bias is a register, and eight rows of a unit are one 16-byte
+// store (MN-major operand: 8 x 8 core matrices 1,024 bytes apart along k, 128
+// along the rows).  Each CTA writes its half of the hidden activations to its
+// own and, with asynchronous stores that complete bytes on the other's
+// barrier, to its partner's operand.  The output layer of tile i runs on CTA
+// i % 2, rows as M = 64 (row r in lane 32 (r / 16) + r % 16).
+//
+// Warps: 0-3 first layer's epilogue, 4-7 second's, 8-11 outputs, 12-19 the
+// observation rows (fp32 loads in row order, 16-bit operand out: no tiling
+// pass over the batch), 20 issues the MMAs.  Persistent over the tiles of its
+// agent: while tile i's first layer runs, tile i - 1 is in its second and
+// i - 2 in its third.  Products, their order along k and every rounding are
+// those of k_tc_forward: the same bits.
+#include <algorithm>
+#include <cstring>
+
+#include "fr_env_dev.cuh"
+#include "fr_ptx.cuh"
+#include "fr_tc.cuh"
+
+namespace fr {
+
+namespace {
+
+constexpr int WD_ROWS = 64;                       // most rows of a tile
+constexpr int WD_UNITS = 128;                     // units per CTA
+constexpr int WD_LOADERS = 8;                     // warps loading observations
+constexpr int WD_MMA_WARP = 12 + WD_LOADERS;
+constexpr int WD_THREADS = 32 * (WD_MMA_WARP + 1);
+constexpr uint32_t WD_XCOL = WD_ROWS * 16u;       // bytes between 8-column chunks of X
+constexpr int WD_GROUP = 4;                       // rows a loader warp stages at a time: 16 ld bytes apart, so
+                                                  // every group of an aligned batch starts on a 16-byte boundary
+constexpr uint32_t WD_H = 256u * WD_ROWS * 2u;    // a hidden operand, 256 units
+constexpr uint32_t WD_ACC2 = 64u, WD_OUT = 128u, WD_W1 = 160u;   // tensor memory columns
+
+struct WdArgs {
+    TcPlan plan;
+    const uint8_t *img;
+    const float *bias;
+    unsigned *err;
+    const float *obs;
+    int ld, rows;
+    float *y;
+    int pair, n, tiles, nan0;                     // CTAs per agent, rows per tile, tiles of the batch
+    uint32_t x_bytes, stage_bytes, w3, x, h1, h2, stage, bars;   // shared memory
+    int bulk;                                     // rows are packed and 16-byte aligned: bulk copies
+};
+
+struct WdBars {
+    uint64_t x_full[2], x_empty[2];               // observations of a tile in / read
+    uint64_t a1_full, a1_free, a2_full, a2_free;  // the layers' accumulators
+    uint64_t h1_full[2], h1_free[2];              // hidden operands: both halves in / read by both CTAs
+    uint64_t h2_full, h2_free[2];                 // h2_free[o]: read by owner o's output layer
+    uint64_t o_full, o_free;
+    uint64_t stage[WD_LOADERS];                   // a loader warp's rows in its stage
+    uint64_t drain;
+    uint32_t tmem;
+    int abort;
+};
+
+__device__ __forceinline__ void wd_wait(uint64_t *bar, uint32_t parity, bool remote, volatile int *abort,
+                                        unsigned *err, unsigned code)
+{
+    if (remote) {
+        if (__all_sync(0xffffffffu, ptx::mbar_try_wait_cluster(bar, parity))) return;
+        ptx::warp_wait_all(bar, parity, true, abort, err, code, TC_WAIT_NS);
+    } else {
+        quick_wait(bar, parity, abort, err, code);
+    }
+}
+
+template <bool NAN0>
+__device__ __forceinline__ void wd_epilogue(const WdArgs &a, WdBars *bars, uint8_t *base, uint32_t tmem, int layer,
+                                            int c, int agent, int count)
+{
+    // layer 0 or 1: accumulators -> the next layer's operand
+    using namespace ptx;
+    const int q = (threadIdx.x >> 5) & 3, lane = threadIdx.x & 31, n = a.n;
+    const bool pair = a.pair == 2, f16 = a.plan.f16 != 0;
+    volatile int *abort = &bars->abort;
+    const int unit = c * WD_UNITS + q * 32 + lane;
+    const float bias = a.bias[((size_t)agent * MAX_LAYERS + layer) * 256 + unit];
+    const uint32_t acc = tmem + (layer ? WD_ACC2 : 0u) + ((uint32_t)(q * 32) << 16);
+    uint64_t *full = layer ? &bars->a2_full : &bars->a1_full, *freeb = layer ? &bars->a2_free : &bars->a1_free;
+    const uint32_t row = (uint32_t)(unit / 8) * 1024u + (uint32_t)(unit % 8) * 16u;
+    const uint32_t other = (uint32_t)(c ^ 1);
+    const uint32_t half_bytes = (uint32_t)(WD_UNITS * n * 2);      // the other CTA's half
+    const uint32_t r_h1 = pair ? map_shared_rank(smem_u32(base + a.h1), other) : 0u;
+    const uint32_t r_h2 = pair ? map_shared_rank(smem_u32(base + a.h2), other) : 0u;
+    for (int i = 0; i < count; ++i) {
+        quick_wait(full, (uint32_t)i & 1u, abort, a.err, 16u);
+        tc_fence_after();
+        const int o = pair ? i & 1 : 0;                            // the tile's output layer runs on CTA o
+        bool mine = true;
+        uint32_t at, rat = 0u, rbar = 0u;
+        uint64_t *ready;
+        if (layer == 0) {
+            const int b = i & 1;
+            if (i >= 2) wd_wait(&bars->h1_free[b], (uint32_t)((i >> 1) - 1) & 1u, pair, abort, a.err, 64u);
+            at = smem_u32(base + a.h1) + (uint32_t)b * WD_H + row;
+            ready = &bars->h1_full[b];
+            if (pair) {
+                rat = r_h1 + (uint32_t)b * WD_H + row;
+                rbar = map_shared_rank(smem_u32(ready), other);
+            }
+        } else {
+            // the second layer has read its operand: both CTAs may refill it
+            if (i + 2 < count && q == 0 && lane == 0) {
+                mbar_arrive(&bars->h1_free[i & 1]);
+                if (pair) mbar_arrive_remote(map_shared_rank(smem_u32(&bars->h1_free[i & 1]), other));
+            }
+            __syncwarp();
+            const int k = pair ? i >> 1 : i;
+            if (k >= 1) wd_wait(&bars->h2_free[o], (uint32_t)(k - 1) & 1u, pair, abort, a.err, 64u);
+            mine = o == c;
+            at = smem_u32(base + a.h2) + row;
+            ready = &bars->h2_full;
+            if (pair && !mine) {
+                rat = r_h2 + row;
+                rbar = map_shared_rank(smem_u32(ready), other);
+            }
+        }
+        const bool remote = rat != 0u;
+        unit_rows<NAN0>(
+            acc, bias, n, f16,
+            [&](int g, const uint32_t *w) {
+                if (mine) st_shared_v4(at + (uint32_t)g * 128u, w[0], w[1], w[2], w[3]);
+                if (remote) st_async_v4(rat + (uint32_t)g * 128u, w[0], w[1], w[2], w[3], rbar);
+            },
+            [&] {
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(freeb);
+            });
+        if (mine) {
+            fence_proxy_async_smem();
+            __syncwarp();
+            if (lane == 0) {
+                if (q == 0 && pair)
+                    mbar_arrive_expect_tx(ready, half_bytes);
+                else
+                    mbar_arrive(ready);
+            }
+        }
+        __syncwarp();
+    }
+}
+
+__global__ void __launch_bounds__(WD_THREADS, 1) k_wide(const __grid_constant__ WdArgs a)
+{
+    using namespace ptx;
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t *base = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    const TcPlan &p = a.plan;
+    const TcLayer &l1 = p.layer[0], &l2 = p.layer[1], &l3 = p.layer[2];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const bool pair = a.pair == 2, f16 = p.f16 != 0;
+    const int n = a.n;
+    const int c = pair ? (int)cluster_ctarank() : 0;
+    const int cl = (int)blockIdx.x / a.pair;
+    const int agent = cl % p.M, first = cl / p.M, stride = ((int)gridDim.x / a.pair) / p.M;
+    const int count = first < a.tiles ? (a.tiles - 1 - first) / stride + 1 : 0;
+    const int owned = pair ? (count + 1 - c) / 2 : count;        // tiles whose output layer runs here
+    WdBars *bars = (WdBars *)(base + a.bars);
+    volatile int *abort = &bars->abort;
+
+    if (threadIdx.x == 0) {
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(&bars->x_full[b], WD_LOADERS);
+            mbar_init(&bars->x_empty[b], 1);
+            mbar_init(&bars->h1_full[b], 4);
+            mbar_init(&bars->h1_free[b], (uint32_t)a.pair);
+            mbar_init(&bars->h2_free[b], 1);
+        }
+        mbar_init(&bars->a1_full, 1);
+        mbar_init(&bars->a1_free, 4);
+        mbar_init(&bars->a2_full, 1);
+        mbar_init(&bars->a2_free, 4);
+        mbar_init(&bars->h2_full, 4);
+        mbar_init(&bars->o_full, 1);
+        mbar_init(&bars->o_free, 4);
+        for (int w = 0; w < WD_LOADERS; ++w) mbar_init(&bars->stage[w], 1);
+        mbar_init(&bars->drain, 1);
+        bars->abort = 0;
+        fence_mbar_init();
+    }
+    if (warp == WD_MMA_WARP) {
+        __syncwarp();
+        tmem_alloc(&bars->tmem, 512u);
+        tmem_relinquish();
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = bars->tmem;
+    const uint32_t w1t = tmem + WD_W1, w2t = w1t + (uint32_t)l1.K / 2u;
+    const int ksteps1 = l1.K / 16, ksteps2 = l2.K / 16, ksteps3 = l3.K / 16;
+
+    // A loader warp stages its groups of rows (g, g + 8, .. of every tile) one
+    // after another; the next one's copy is issued as soon as the stage is read.
+    float *stage = (float *)(base + a.stage + (uint32_t)(warp - 12) * a.stage_bytes);   // loader warps only
+    auto stage_group = [&](int i, int g) {
+        const int row = (first + i * stride) * n + g * WD_GROUP;
+        const int have = max(0, min(WD_GROUP, a.rows - row));
+        if (a.bulk && have == WD_GROUP) {
+            if (lane == 0) {
+                mbar_arrive_expect_tx(&bars->stage[warp - 12], (uint32_t)(l1.fin * 16));
+                bulk_g2s(stage, a.obs + (int64_t)row * a.ld, (uint32_t)(l1.fin * 16), &bars->stage[warp - 12]);
+            }
+            return true;
+        }
+        for (int r = 0; r < WD_GROUP; ++r)
+#pragma unroll 4
+            for (int k = lane; k < l1.fin; k += 32)
+                stage[r * l1.fin + k] = r < have ? __ldg(a.obs + (int64_t)(row + r) * a.ld + k) : 0.0f;
+        __syncwarp();
+        return false;
+    };
+    grid_launch_next();
+    const int groups = n / WD_GROUP;
+    bool staged = false;                                   // the stage's rows come by a bulk copy
+    if (warp >= 12 && warp < WD_MMA_WARP && warp - 12 < groups) staged = stage_group(0, warp - 12);
+
+    if (warp < 12) {
+        // this CTA's units of the first two layers into tensor memory, lane =
+        // unit, the two 16-byte core rows of a K = 16 step into eight columns;
+        // four steps' loads in flight.  Units past a layer's get zeros.
+        const uint8_t *img = a.img + (size_t)agent * p.agent_bytes;
+        const int q = warp & 3, unit = c * WD_UNITS + q * 32 + lane;
+        const uint32_t lane_off = (uint32_t)(q * 32) << 16;
+        const int all = ksteps1 + ksteps2;
+        for (int s0 = warp >> 2; s0 < all; s0 += 12) {
+            uint4 v[4][2];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int s = s0 + 3 * u;
+                const bool second = s >= ksteps1;
+                const TcLayer &ly = second ? l2 : l1;
+                const int k = second ? s - ksteps1 : s;
+                v[u][0] = v[u][1] = make_uint4(0u, 0u, 0u, 0u);
+                if (s < all && unit < ly.N) {
+                    const uint4 *src = (const uint4 *)(img + ly.off) + (size_t)(2 * k) * ly.N + unit;
+                    v[u][0] = __ldg(src);
+                    v[u][1] = __ldg(src + ly.N);
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int s = s0 + 3 * u;
+                if (s < all) {                             // warp-uniform
+                    const uint32_t w[8] = {v[u][0].x, v[u][0].y, v[u][0].z, v[u][0].w,
+                                           v[u][1].x, v[u][1].y, v[u][1].z, v[u][1].w};
+                    __syncwarp();
+                    tmem_st8(w1t + 8u * (uint32_t)s + lane_off, w);
+                }
+            }
+        }
+        // the output layer's weights
+        const uint4 *src3 = (const uint4 *)(img + l3.off);
+        uint4 *dst3 = (uint4 *)(base + a.w3);
+        for (int i = threadIdx.x; i < l3.N * l3.K / 8; i += 384) dst3[i] = __ldg(src3 + i);
+        // hidden rows past the tile's n are read by the M = 64 output layer
+        uint4 *h2 = (uint4 *)(base + a.h2);
+        for (int i = threadIdx.x; i < (int)(WD_H / 16u); i += 384) h2[i] = make_uint4(0u, 0u, 0u, 0u);
+        tmem_st_wait();
+        fence_proxy_async_smem();
+        tc_fence_before();
+    }
+    if (pair)
+        cluster_sync_all();                                // barriers and zeroed operands of both CTAs
+    else
+        __syncthreads();
+    tc_fence_after();
+
+    if (warp < 8) {
+        const int layer = warp >> 2;
+        if (a.nan0)
+            wd_epilogue<true>(a, bars, base, tmem, layer, c, agent, count);
+        else
+            wd_epilogue<false>(a, bars, base, tmem, layer, c, agent, count);
+    } else if (warp < 12) {
+        // ------------------------------------------------------- outputs
+        const int q = warp & 3, r = q * 16 + lane;
+        const float *b3 = a.bias + ((size_t)agent * MAX_LAYERS + 2) * 256;
+        const float bl = lane < l3.N ? b3[lane] : 0.0f;
+        for (int m = 0; m < owned; ++m) {
+            const int i = pair ? 2 * m + c : m;
+            quick_wait(&bars->o_full, (uint32_t)m & 1u, abort, a.err, 16u);
+            tc_fence_after();
+            if (q == 0 && lane == 0 && i + a.pair < count) {
+                // this CTA's hidden operand may be refilled
+                mbar_arrive(&bars->h2_free[c]);
+                if (pair) mbar_arrive_remote(map_shared_rank(smem_u32(&bars->h2_free[c]), (uint32_t)(c ^ 1)));
+            }
+            uint32_t v[32];
+            __syncwarp();
+            tmem_ld32(tmem + WD_OUT + ((uint32_t)(q * 32) << 16), v);
+            tmem_ld_wait();
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&bars->o_free);
+            const int g = (first + i * stride) * n + r;
+            const bool out = lane < 16 && r < n && g < a.rows;
+            float *yr = a.y + ((size_t)agent * a.rows + g) * l3.fout;
+#pragma unroll
+            for (int k = 0; k < 32; ++k) {
+                const float b = __shfl_sync(FULL_MASK, bl, k);
+                if (k < l3.fout && out) {
+                    const float x = __uint_as_float(v[k]) + b;
+                    yr[k] = p.out_act ? tanhf(x) : x;
+                }
+            }
+        }
+    } else if (warp < WD_MMA_WARP) {
+        // -------------------------------------------------- observations
+        // lane: row lane % 4 of the group, 8-column chunk lane / 4, + 8, ..
+        const int w = warp - 12, r4 = lane & 3;
+        const uint32_t xs = smem_u32(base + a.x);
+        const int fin = l1.fin, chunks = l1.K / 8;
+        uint32_t sph = 0;
+        volatile int no_abort = 0;                         // a copy issued is always waited for
+        for (int i = 0; i < count; ++i) {
+            const int b = i & 1;
+            if (i >= 2) quick_wait(&bars->x_empty[b], (uint32_t)((i >> 1) - 1) & 1u, abort, a.err, 1u);
+            for (int g = w; g < groups; g += WD_LOADERS) {
+                if (staged) {
+                    quick_wait(&bars->stage[w], sph, &no_abort, a.err, 1u);
+                    sph ^= 1u;
+                }
+                const float *src = stage + r4 * fin;
+                const int r = g * WD_GROUP + r4;
+                const uint32_t at = xs + (uint32_t)b * a.x_bytes + (uint32_t)(r / 8) * 128u + (uint32_t)(r % 8) * 16u;
+                for (int ch = lane >> 2; ch < chunks; ch += 8) {
+                    float x[8];
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) x[u] = ch * 8 + u < fin ? src[ch * 8 + u] : 0.0f;
+                    uint32_t v[4];
+                    pack8_16(x, v, f16);
+                    st_shared_v4(at + (uint32_t)ch * WD_XCOL, v[0], v[1], v[2], v[3]);
+                }
+                __syncwarp();                              // the stage has been read
+                if (g + WD_LOADERS < groups)
+                    staged = stage_group(i, g + WD_LOADERS);
+                else if (i + 1 < count)
+                    staged = stage_group(i + 1, w);
+                else
+                    staged = false;
+            }
+            fence_proxy_async_smem();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&bars->x_full[b]);
+        }
+    } else {
+        // ------------------------------------------------------ MMA issue
+        const uint32_t id1 = idesc_16(WD_UNITS, n, f16), id2 = id1 | (1u << 16);
+        const uint32_t id3 = idesc_16(WD_ROWS, l3.N, f16) | (1u << 15);
+        const uint64_t xd = smem_desc(smem_u32(base + a.x), WD_XCOL, 128u);
+        const uint64_t h1d = smem_desc(smem_u32(base + a.h1), 1024u, 128u);
+        const uint64_t h2d = smem_desc(smem_u32(base + a.h2), 1024u, 128u);
+        const uint64_t w3d = smem_desc(smem_u32(base + a.w3), (uint32_t)(l3.N * 16), 128u);
+        int m = 0;
+        // tile t's first layer, tile t - 1's second, tile t - 2's third
+        for (int t = 0; t < count + 2; ++t) {
+            if (t < count) {
+                const int b = t & 1;
+                quick_wait(&bars->x_full[b], (uint32_t)(t >> 1) & 1u, abort, a.err, 2u);
+                if (t >= 1) quick_wait(&bars->a1_free, (uint32_t)(t - 1) & 1u, abort, a.err, 2u);
+                tc_fence_after();
+                if (elect_one()) {
+                    const uint64_t xb = xd + (uint64_t)(((uint32_t)b * a.x_bytes) >> 4);
+                    for (int k = 0; k < ksteps1; ++k)
+                        mma_bf16_ta(tmem, w1t + 8u * (uint32_t)k, xb + (uint64_t)(2u * WD_XCOL / 16u * (uint32_t)k), id1,
+                                    k ? 1u : 0u);
+                    mma_commit(&bars->x_empty[b]);
+                    mma_commit(&bars->a1_full);
+                }
+                __syncwarp();
+            }
+            if (t >= 1 && t - 1 < count) {
+                const int i = t - 1, b = i & 1;
+                wd_wait(&bars->h1_full[b], (uint32_t)(i >> 1) & 1u, pair, abort, a.err, 4u);
+                if (i >= 1) quick_wait(&bars->a2_free, (uint32_t)(i - 1) & 1u, abort, a.err, 2u);
+                fence_proxy_async_smem();                  // the partner's half came by generic stores
+                tc_fence_after();
+                if (elect_one()) {
+                    const uint64_t hb = h1d + (uint64_t)(((uint32_t)b * WD_H) >> 4);
+                    for (int k = 0; k < ksteps2; ++k)
+                        mma_bf16_ta(tmem + WD_ACC2, w2t + 8u * (uint32_t)k, hb + (uint64_t)(128 * k), id2, k ? 1u : 0u);
+                    mma_commit(&bars->a2_full);
+                }
+                __syncwarp();
+            }
+            if (t >= 2 && (!pair || ((t - 2) & 1) == c)) {
+                wd_wait(&bars->h2_full, (uint32_t)m & 1u, pair, abort, a.err, 4u);
+                if (m >= 1) quick_wait(&bars->o_free, (uint32_t)(m - 1) & 1u, abort, a.err, 2u);
+                fence_proxy_async_smem();
+                tc_fence_after();
+                if (elect_one()) {
+                    for (int k = 0; k < ksteps3; ++k)
+                        mma_bf16(tmem + WD_OUT, h2d + (uint64_t)(128 * k), w3d + (uint64_t)(2 * l3.N * k), id3, k ? 1u : 0u);
+                    mma_commit(&bars->o_full);
+                }
+                __syncwarp();
+                ++m;
+            }
+        }
+        // every MMA issued completes before tensor memory is released; the
+        // partner's bytes of the last tiles have landed too (or timed out)
+        if (elect_one()) mma_commit(&bars->drain);
+        __syncwarp();
+        volatile int no_abort = 0;
+        warp_wait_all(&bars->drain, 0u, false, &no_abort, a.err, 128u, TC_WAIT_NS);
+        for (int i = count > 2 ? count - 2 : 0; pair && i < count; ++i)
+            warp_wait_all(&bars->h1_full[i & 1], (uint32_t)(i >> 1) & 1u, true, &no_abort, a.err, 8u, TC_WAIT_NS);
+        if (pair && owned > 0)
+            warp_wait_all(&bars->h2_full, (uint32_t)(owned - 1) & 1u, true, &no_abort, a.err, 8u, TC_WAIT_NS);
+    }
+    __syncwarp();
+    tc_fence_before();
+    __syncthreads();
+    if (warp == WD_MMA_WARP) {
+        __syncwarp();
+        tc_fence_after();
+        tmem_dealloc(tmem, 512u);
+    }
+    __syncwarp();
+    if (pair) cluster_sync_all();                          // no peer touches this CTA's memory after it exits
+}
+
+// Shared memory of a launch (bytes, without the alignment slack).
+uint32_t wd_layout(const TcPlan &p, WdArgs *a)
+{
+    uint32_t off = 0;
+    auto take = [&](uint32_t bytes) {
+        const uint32_t at = off;
+        off += (bytes + 127u) & ~127u;
+        return at;
+    };
+    const uint32_t x_bytes = (uint32_t)(p.layer[0].K / 8) * WD_XCOL;
+    const uint32_t stage_bytes = (uint32_t)(WD_GROUP * 4 * p.layer[0].fin);
+    const uint32_t h2 = take(WD_H), h1 = take(2u * WD_H), x = take(2u * x_bytes);
+    const uint32_t w3 = take((uint32_t)(p.layer[2].N * p.layer[2].K) * 2u), stage = take(WD_LOADERS * stage_bytes);
+    const uint32_t bars = take(sizeof(WdBars));
+    if (a) {
+        a->x_bytes = x_bytes;
+        a->stage_bytes = stage_bytes;
+        a->stage = stage;
+        a->h1 = h1;
+        a->h2 = h2;
+        a->x = x;
+        a->w3 = w3;
+        a->bars = bars;
+    }
+    return off;
+}
+
+}  // namespace
+
+// Networks k_wide takes: tensor memory must hold the first layer's weights.
+bool wd_ok(const fr_ensemble *e)
+{
+    if (!e->tc) return false;
+    const TcPlan &p = e->tc->plan;
+    return p.esz == 2 && p.split == 1 && p.L == 3 && p.layer[0].K <= 304 && p.layer[0].N <= 256 &&
+           p.layer[1].N <= 256 && p.layer[1].K <= 256 && p.layer[2].K <= 256 && p.layer[2].N <= 32;
+}
+
+int wd_forward(const fr_ensemble *e, const float *obs, int ld, int n, float *y, cudaStream_t s)
+{
+    const TcPlan &p = e->tc->plan;
+    WdArgs a;
+    memset(&a, 0, sizeof(a));
+    a.plan = p;
+    a.img = e->tc->img;
+    a.bias = e->tc->bias;
+    a.err = e->tc->err;
+    a.obs = obs;
+    a.ld = ld;
+    a.rows = n;
+    a.y = y;
+    a.nan0 = tc_small_batch(e, n);
+    a.bulk = ld == p.layer[0].fin && ((uintptr_t)obs & 15u) == 0;
+    a.pair = p.layer[0].N > WD_UNITS || p.layer[1].N > WD_UNITS ? 2 : 1;
+    const uint32_t smem = wd_layout(p, &a) + 1024u;
+    // tiles: as few rows each as spread the batch over every cluster in the
+    // waves it needs anyway
+    const int64_t per_agent = std::max(1, e->ctx->sm_count / a.pair / p.M);
+    const int64_t waves = (n + WD_ROWS * per_agent - 1) / (WD_ROWS * per_agent);
+    const int64_t per = (n + waves * per_agent - 1) / (waves * per_agent);
+    a.n = (int)std::min<int64_t>(WD_ROWS, (per + 15) / 16 * 16);
+    a.tiles = (int)ceil_div(n, a.n);
+    FR_CUDA(set_max_smem_once((const void *)k_wide, e->ctx->device));
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(a.pair * p.M * (int)std::min<int64_t>(per_agent, a.tiles)), 1, 1);
+    cfg.blockDim = dim3(WD_THREADS, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)a.pair;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    FR_CUDA(cudaLaunchKernelEx(&cfg, k_wide, a));
+    return FR_OK;
+}
+
+}  // namespace fr
