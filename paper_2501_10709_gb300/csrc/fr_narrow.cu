@@ -298,7 +298,7 @@ __global__ void __launch_bounds__(32 * (4 * NW_MAX_AGENTS + 4), 1) k_narrow(cons
     const NwShape &sh = a.sh;
     const TcPlan &p = a.plan;
     const int M = sh.M, n = sh.n;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = (int)uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
     const int j = warp >> 2, q = warp & 3;       // agent (M: the rows' warps), TMEM lane quarter
     NwBars *bars = (NwBars *)(base + sh.bars);
     volatile int *abort = &bars->abort;
@@ -350,7 +350,7 @@ __global__ void __launch_bounds__(32 * (4 * NW_MAX_AGENTS + 4), 1) k_narrow(cons
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = bars->tmem;
+    const uint32_t tmem = uniform(bars->tmem);
     if (j < sh.ntm) {
         const uint32_t w2 = tmem + 64u * (uint32_t)(M + j) + ((uint32_t)(q * 32) << 16);
 #pragma unroll 2

@@ -166,7 +166,7 @@ __global__ void __launch_bounds__(WD_THREADS, 1) k_wide(const __grid_constant__ 
     uint8_t *base = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     const TcPlan &p = a.plan;
     const TcLayer &l1 = p.layer[0], &l2 = p.layer[1], &l3 = p.layer[2];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = (int)uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
     const bool pair = a.pair == 2, f16 = p.f16 != 0;
     const int n = a.n;
     const int c = pair ? (int)cluster_ctarank() : 0;
@@ -205,7 +205,7 @@ __global__ void __launch_bounds__(WD_THREADS, 1) k_wide(const __grid_constant__ 
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = bars->tmem;
+    const uint32_t tmem = uniform(bars->tmem);
     const uint32_t w1t = tmem + WD_W1, w2t = w1t + (uint32_t)l1.K / 2u;
     const int ksteps1 = l1.K / 16, ksteps2 = l2.K / 16, ksteps3 = l3.K / 16;
 
