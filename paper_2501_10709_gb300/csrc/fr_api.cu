@@ -1021,6 +1021,7 @@ int ensemble_act(const fr_ensemble *e, const float *obs, int32_t n, void *act, v
     int rc = use_device(e->ctx);
     if (rc) return rc;
     cudaStream_t s = (cudaStream_t)stream;
+    if (wd_act_ok(e, n)) return wd_act(e, obs, n, (float *)act, s);
     const int out = e->dims[e->L];
     float *y = nullptr;
     FR_CUDA(cudaMallocAsync((void **)&y, 4ull * e->M * n * out, s));

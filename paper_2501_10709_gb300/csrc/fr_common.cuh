@@ -376,6 +376,9 @@ int nw_forward(const fr_ensemble *e, const float *obs, int ld, int n, float *y, 
 // two hidden layers up to 256 wide, weights resident in CTA pairs (fr_wide.cu)
 bool wd_ok(const fr_ensemble *e);
 int wd_forward(const fr_ensemble *e, const float *obs, int ld, int n, float *y, cudaStream_t s);
+// the weighted mean of the agents' outputs in the same launch, for batches wd_act_ok takes
+bool wd_act_ok(const fr_ensemble *e, int n);
+int wd_act(const fr_ensemble *e, const float *obs, int n, float *act, cudaStream_t s);
 // Fewer 128-row tiles than SMs.  Hidden NaNs become 0 (max(x, 0)) in such
 // batches and stay NaN in larger ones.
 inline int tc_small_batch(const fr_ensemble *e, int n) { return (int)ceil_div(n, 128) < e->ctx->sm_count; }

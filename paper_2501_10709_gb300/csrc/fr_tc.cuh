@@ -172,6 +172,7 @@ __device__ __forceinline__ void unit_rows(uint32_t acc, float bias, int n, bool 
     uint64_t b2;
     asm("mov.b64 %0, {%1, %1};" : "=l"(b2) : "f"(bias));
     int c0 = 0;
+#pragma unroll 1
     for (; c0 + 32 <= n; c0 += 32) {
         uint32_t v[32];
         __syncwarp();

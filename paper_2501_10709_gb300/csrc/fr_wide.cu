@@ -18,14 +18,34 @@
 // barrier, to its partner's operand.  The output layer of tile i runs on CTA
 // i % 2, rows as M = 64 (row r in lane 32 (r / 16) + r % 16).
 //
+// ensemble_act on a small batch runs the agents' pairs as one cluster: the
+// others send their outputs to agent 0's CTAs, which write the weighted mean
+// (no per-agent outputs in memory, no second launch, no allocation).
+//
 // Warps: 0-3 first layer's epilogue, 4-7 second's, 8-11 outputs, 12-19 the
 // observation rows (fp32 loads in row order, 16-bit operand out: no tiling
 // pass over the batch), 20 issues the MMAs.  Persistent over the tiles of its
 // agent: while tile i's first layer runs, tile i - 1 is in its second and
 // i - 2 in its third.  Products, their order along k and every rounding are
 // those of k_tc_forward: the same bits.
+//
+// Measured on 3 x 301-256-256-30 (whole calls; before: k_tc_forward below
+// 19,456 rows, a tiling pass and k_tc_actor2 above): ensemble_act on 8 rows
+// 43.1 -> 12.0 us, on 2,048 rows 51.3 -> 17.4 us; ensemble_forward on 77,824
+// rows 151 -> 127 us.  A tile of 64 rows takes about 4,700 cycles there, of
+// which the tensor pipe works 1,500: a K = 16 step of 64 rows is 32 cycles of
+// MMA but 45 to 70 of issue (its operands go to uniform registers one by one,
+// and the code of 21 warps in five roles does not stay in the instruction
+// caches: unrolling the issue loops made it slower, compile-time strides
+// faster), and the loader's conversion and copies take as long as both layers.
+// Small batches are bound by the chain of three layers with an exchange
+// between CTAs after each of the first two (about 5,500 cycles), behind the
+// weights' 143 KB per SM.
 #include <algorithm>
 #include <cstring>
+#include <map>
+#include <mutex>
+#include <utility>
 
 #include "fr_env_dev.cuh"
 #include "fr_ptx.cuh"
@@ -36,14 +56,15 @@ namespace fr {
 namespace {
 
 constexpr int WD_ROWS = 64;                       // most rows of a tile
+constexpr int WD_OUTS = 32;                       // outputs, padded
 constexpr int WD_UNITS = 128;                     // units per CTA
 constexpr int WD_LOADERS = 8;                     // warps loading observations
 constexpr int WD_MMA_WARP = 12 + WD_LOADERS;
 constexpr int WD_THREADS = 32 * (WD_MMA_WARP + 1);
-constexpr uint32_t WD_XCOL = WD_ROWS * 16u;       // bytes between 8-column chunks of X
 constexpr int WD_GROUP = 4;                       // rows a loader warp stages at a time: 16 ld bytes apart, so
                                                   // every group of an aligned batch starts on a 16-byte boundary
-constexpr uint32_t WD_H = 256u * WD_ROWS * 2u;    // a hidden operand, 256 units
+constexpr int WD_ACT_MAX = 4096;                  // most rows combined in the same launch
+constexpr int WD_ACT_ROWS = 48;                   // most rows of a tile where the agents are combined
 constexpr uint32_t WD_ACC2 = 64u, WD_OUT = 128u, WD_W1 = 160u;   // tensor memory columns
 
 struct WdArgs {
@@ -55,7 +76,9 @@ struct WdArgs {
     int ld, rows;
     float *y;
     int pair, n, tiles, nan0;                     // CTAs per agent, rows per tile, tiles of the batch
-    uint32_t x_bytes, stage_bytes, w3, x, h1, h2, stage, bars;   // shared memory
+    int act;                                      // 1: y is the weighted mean of the agents [rows][outputs]
+    float w[MAX_AGENTS];
+    uint32_t x_bytes, h_bytes, stage_bytes, w3, x, h1, h2, stage, comb, bars;   // shared memory
     int bulk;                                     // rows are packed and 16-byte aligned: bulk copies
 };
 
@@ -65,6 +88,7 @@ struct WdBars {
     uint64_t h1_full[2], h1_free[2];              // hidden operands: both halves in / read by both CTAs
     uint64_t h2_full, h2_free[2];                 // h2_free[o]: read by owner o's output layer
     uint64_t o_full, o_free;
+    uint64_t comb_full, comb_free;                // the other agents' outputs in / read
     uint64_t stage[WD_LOADERS];                   // a loader warp's rows in its stage
     uint64_t drain;
     uint32_t tmem;
@@ -82,21 +106,21 @@ __device__ __forceinline__ void wd_wait(uint64_t *bar, uint32_t parity, bool rem
     }
 }
 
-template <bool NAN0>
+template <int n, bool NAN0>
 __device__ __forceinline__ void wd_epilogue(const WdArgs &a, WdBars *bars, uint8_t *base, uint32_t tmem, int layer,
-                                            int c, int agent, int count)
+                                            int c, int rank, int agent, int count)
 {
     // layer 0 or 1: accumulators -> the next layer's operand
     using namespace ptx;
-    const int q = (threadIdx.x >> 5) & 3, lane = threadIdx.x & 31, n = a.n;
+    const int q = (threadIdx.x >> 5) & 3, lane = threadIdx.x & 31;
     const bool pair = a.pair == 2, f16 = a.plan.f16 != 0;
     volatile int *abort = &bars->abort;
     const int unit = c * WD_UNITS + q * 32 + lane;
     const float bias = a.bias[((size_t)agent * MAX_LAYERS + layer) * 256 + unit];
     const uint32_t acc = tmem + (layer ? WD_ACC2 : 0u) + ((uint32_t)(q * 32) << 16);
     uint64_t *full = layer ? &bars->a2_full : &bars->a1_full, *freeb = layer ? &bars->a2_free : &bars->a1_free;
-    const uint32_t row = (uint32_t)(unit / 8) * 1024u + (uint32_t)(unit % 8) * 16u;
-    const uint32_t other = (uint32_t)(c ^ 1);
+    const uint32_t row = (uint32_t)(unit / 8) * (uint32_t)(n * 16) + (uint32_t)(unit % 8) * 16u;
+    const uint32_t other = (uint32_t)(rank ^ 1);
     const uint32_t half_bytes = (uint32_t)(WD_UNITS * n * 2);      // the other CTA's half
     const uint32_t r_h1 = pair ? map_shared_rank(smem_u32(base + a.h1), other) : 0u;
     const uint32_t r_h2 = pair ? map_shared_rank(smem_u32(base + a.h2), other) : 0u;
@@ -110,10 +134,10 @@ __device__ __forceinline__ void wd_epilogue(const WdArgs &a, WdBars *bars, uint8
         if (layer == 0) {
             const int b = i & 1;
             if (i >= 2) wd_wait(&bars->h1_free[b], (uint32_t)((i >> 1) - 1) & 1u, pair, abort, a.err, 64u);
-            at = smem_u32(base + a.h1) + (uint32_t)b * WD_H + row;
+            at = smem_u32(base + a.h1) + (uint32_t)b * a.h_bytes + row;
             ready = &bars->h1_full[b];
             if (pair) {
-                rat = r_h1 + (uint32_t)b * WD_H + row;
+                rat = r_h1 + (uint32_t)b * a.h_bytes + row;
                 rbar = map_shared_rank(smem_u32(ready), other);
             }
         } else {
@@ -159,6 +183,62 @@ __device__ __forceinline__ void wd_epilogue(const WdArgs &a, WdBars *bars, uint8
     }
 }
 
+// Owned tile m's accumulators v of row r (bl: lane k's bias of output k):
+// agents 1 .. send their rows' outputs to agent 0's CTA of the same half,
+// which forms the weighted mean.
+__device__ __forceinline__ void wd_combine(const WdArgs &a, WdBars *bars, uint8_t *base, const uint32_t (&v)[32], float bl,
+                                        int n, int r, int c, int agent, int m, int owned, float *yr)
+{
+    using namespace ptx;
+    const TcPlan &p = a.plan;
+    const int fout = p.layer[2].fout, lane = threadIdx.x & 31;
+    volatile int *abort = &bars->abort;
+    const uint32_t comb = smem_u32(base + a.comb);
+    uint32_t far = 0u, far_bar = 0u;
+    if (agent > 0) {
+        far = map_shared_rank(comb, (uint32_t)c) + (uint32_t)(((agent - 1) * n + r) * 128);
+        far_bar = map_shared_rank(smem_u32(&bars->comb_full), (uint32_t)c);
+        if (m > 0) wd_wait(&bars->comb_free, (uint32_t)(m - 1) & 1u, true, abort, a.err, 64u);
+    } else if (p.M > 1) {
+        wd_wait(&bars->comb_full, (uint32_t)m & 1u, true, abort, a.err, 64u);
+    }
+#pragma unroll
+    for (int k0 = 0; k0 < 32; k0 += 4) {
+        float x[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            x[u] = __uint_as_float(v[k0 + u]) + __shfl_sync(FULL_MASK, bl, k0 + u);
+            if (p.out_act && k0 + u < fout) x[u] = tanhf(x[u]);
+        }
+        if (agent > 0) {
+            if (lane < 16 && r < n)
+                st_async_v4(far + (uint32_t)(k0 * 4), __float_as_uint(x[0]), __float_as_uint(x[1]),
+                            __float_as_uint(x[2]), __float_as_uint(x[3]), far_bar);
+        } else if (yr) {
+            // a_0 + sum w_j (a_j - a_0), rounded at every operation
+            float acc[4] = {x[0], x[1], x[2], x[3]};
+            for (int j = 1; j < p.M; ++j) {
+                const uint4 o = ld_shared_v4(comb + (uint32_t)(((j - 1) * n + r) * 128 + k0 * 4));
+                const uint32_t ou[4] = {o.x, o.y, o.z, o.w};
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    acc[u] = __fadd_rn(acc[u], __fmul_rn(a.w[j], __fsub_rn(__uint_as_float(ou[u]), x[u])));
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (k0 + u < fout) yr[k0 + u] = acc[u];
+        }
+    }
+    __syncwarp();
+    if (agent == 0 && m + 1 < owned && lane < p.M - 1)
+        mbar_arrive_remote(map_shared_rank(smem_u32(&bars->comb_free), (uint32_t)((lane + 1) * a.pair + c)));
+    __syncwarp();
+}
+
+// n: rows per tile, at compile time: descriptors that advance by constants cost
+// the issuing warp less than its MMAs (77,824 rows: 139 us, 153 us with n a
+// parameter).
+template <int n>
 __global__ void __launch_bounds__(WD_THREADS, 1) k_wide(const __grid_constant__ WdArgs a)
 {
     using namespace ptx;
@@ -168,10 +248,12 @@ __global__ void __launch_bounds__(WD_THREADS, 1) k_wide(const __grid_constant__ 
     const TcLayer &l1 = p.layer[0], &l2 = p.layer[1], &l3 = p.layer[2];
     const int warp = (int)uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
     const bool pair = a.pair == 2, f16 = p.f16 != 0;
-    const int n = a.n;
-    const int c = pair ? (int)cluster_ctarank() : 0;
-    const int cl = (int)blockIdx.x / a.pair;
-    const int agent = cl % p.M, first = cl / p.M, stride = ((int)gridDim.x / a.pair) / p.M;
+    const int size = a.pair * (a.act ? p.M : 1);                // CTAs of the cluster
+    const int rank = size > 1 ? (int)cluster_ctarank() : 0, c = pair ? rank & 1 : 0;
+    const int cl = (int)blockIdx.x / size, clusters = (int)gridDim.x / size;
+    // a cluster is one agent's, or every agent's where their outputs are combined
+    const int agent = a.act ? rank / a.pair : cl % p.M, first = a.act ? cl : cl / p.M;
+    const int stride = a.act ? clusters : clusters / p.M;
     const int count = first < a.tiles ? (a.tiles - 1 - first) / stride + 1 : 0;
     const int owned = pair ? (count + 1 - c) / 2 : count;        // tiles whose output layer runs here
     WdBars *bars = (WdBars *)(base + a.bars);
@@ -192,6 +274,8 @@ __global__ void __launch_bounds__(WD_THREADS, 1) k_wide(const __grid_constant__ 
         mbar_init(&bars->h2_full, 4);
         mbar_init(&bars->o_full, 1);
         mbar_init(&bars->o_free, 4);
+        mbar_init(&bars->comb_full, 1);
+        mbar_init(&bars->comb_free, 4);
         for (int w = 0; w < WD_LOADERS; ++w) mbar_init(&bars->stage[w], 1);
         mbar_init(&bars->drain, 1);
         bars->abort = 0;
@@ -232,7 +316,10 @@ __global__ void __launch_bounds__(WD_THREADS, 1) k_wide(const __grid_constant__ 
     grid_launch_next();
     const int groups = n / WD_GROUP;
     bool staged = false;                                   // the stage's rows come by a bulk copy
-    if (warp >= 12 && warp < WD_MMA_WARP && warp - 12 < groups) staged = stage_group(0, warp - 12);
+    if (warp >= 12 && warp < WD_MMA_WARP) {
+        grid_wait_previous();                              // whatever wrote the observations
+        if (warp - 12 < groups) staged = stage_group(0, warp - 12);
+    }
 
     if (warp < 12) {
         // this CTA's units of the first two layers into tensor memory, lane =
@@ -268,19 +355,19 @@ __global__ void __launch_bounds__(WD_THREADS, 1) k_wide(const __grid_constant__ 
                 }
             }
         }
-        // the output layer's weights
+        // the output layer's weights, padded to 32 outputs
         const uint4 *src3 = (const uint4 *)(img + l3.off);
         uint4 *dst3 = (uint4 *)(base + a.w3);
-        for (int i = threadIdx.x; i < l3.N * l3.K / 8; i += 384) dst3[i] = __ldg(src3 + i);
-        // hidden rows past the tile's n are read by the M = 64 output layer
-        uint4 *h2 = (uint4 *)(base + a.h2);
-        for (int i = threadIdx.x; i < (int)(WD_H / 16u); i += 384) h2[i] = make_uint4(0u, 0u, 0u, 0u);
+        for (int i = threadIdx.x; i < 32 * l3.K / 8; i += 384) {
+            const int k = i >> 5, row = i & 31;
+            dst3[i] = row < l3.N ? __ldg(src3 + (size_t)k * l3.N + row) : make_uint4(0u, 0u, 0u, 0u);
+        }
         tmem_st_wait();
         fence_proxy_async_smem();
         tc_fence_before();
     }
-    if (pair)
-        cluster_sync_all();                                // barriers and zeroed operands of both CTAs
+    if (size > 1)
+        cluster_sync_all();                                // the barriers of every CTA
     else
         __syncthreads();
     tc_fence_after();
@@ -288,22 +375,25 @@ __global__ void __launch_bounds__(WD_THREADS, 1) k_wide(const __grid_constant__ 
     if (warp < 8) {
         const int layer = warp >> 2;
         if (a.nan0)
-            wd_epilogue<true>(a, bars, base, tmem, layer, c, agent, count);
+            wd_epilogue<n, true>(a, bars, base, tmem, layer, c, rank, agent, count);
         else
-            wd_epilogue<false>(a, bars, base, tmem, layer, c, agent, count);
+            wd_epilogue<n, false>(a, bars, base, tmem, layer, c, rank, agent, count);
     } else if (warp < 12) {
         // ------------------------------------------------------- outputs
         const int q = warp & 3, r = q * 16 + lane;
         const float *b3 = a.bias + ((size_t)agent * MAX_LAYERS + 2) * 256;
         const float bl = lane < l3.N ? b3[lane] : 0.0f;
+        grid_wait_previous();                              // whatever still reads the outputs
         for (int m = 0; m < owned; ++m) {
             const int i = pair ? 2 * m + c : m;
+            if (n <= WD_ACT_ROWS && a.act && agent == 0 && p.M > 1 && q == 0 && lane == 0)
+                mbar_arrive_expect_tx(&bars->comb_full, (uint32_t)((p.M - 1) * n * 128));
             quick_wait(&bars->o_full, (uint32_t)m & 1u, abort, a.err, 16u);
             tc_fence_after();
             if (q == 0 && lane == 0 && i + a.pair < count) {
                 // this CTA's hidden operand may be refilled
                 mbar_arrive(&bars->h2_free[c]);
-                if (pair) mbar_arrive_remote(map_shared_rank(smem_u32(&bars->h2_free[c]), (uint32_t)(c ^ 1)));
+                if (pair) mbar_arrive_remote(map_shared_rank(smem_u32(&bars->h2_free[c]), (uint32_t)(rank ^ 1)));
             }
             uint32_t v[32];
             __syncwarp();
@@ -314,13 +404,17 @@ __global__ void __launch_bounds__(WD_THREADS, 1) k_wide(const __grid_constant__ 
             if (lane == 0) mbar_arrive(&bars->o_free);
             const int g = (first + i * stride) * n + r;
             const bool out = lane < 16 && r < n && g < a.rows;
-            float *yr = a.y + ((size_t)agent * a.rows + g) * l3.fout;
+            if (n <= WD_ACT_ROWS && a.act) {               // (its code stays out of the tallest tiles' kernel)
+                wd_combine(a, bars, base, v, bl, n, r, c, agent, m, owned, out ? a.y + (size_t)g * l3.fout : nullptr);
+            } else {
+                float *yr = a.y + ((size_t)agent * a.rows + g) * l3.fout;
 #pragma unroll
-            for (int k = 0; k < 32; ++k) {
-                const float b = __shfl_sync(FULL_MASK, bl, k);
-                if (k < l3.fout && out) {
-                    const float x = __uint_as_float(v[k]) + b;
-                    yr[k] = p.out_act ? tanhf(x) : x;
+                for (int k = 0; k < 32; ++k) {
+                    const float b = __shfl_sync(FULL_MASK, bl, k);
+                    if (k < l3.fout && out) {
+                        const float x = __uint_as_float(v[k]) + b;
+                        yr[k] = p.out_act ? tanhf(x) : x;
+                    }
                 }
             }
         }
@@ -330,6 +424,7 @@ __global__ void __launch_bounds__(WD_THREADS, 1) k_wide(const __grid_constant__ 
         const int w = warp - 12, r4 = lane & 3;
         const uint32_t xs = smem_u32(base + a.x);
         const int fin = l1.fin, chunks = l1.K / 8;
+        const uint32_t xcol = (uint32_t)(n * 16);
         uint32_t sph = 0;
         volatile int no_abort = 0;                         // a copy issued is always waited for
         for (int i = 0; i < count; ++i) {
@@ -349,7 +444,7 @@ __global__ void __launch_bounds__(WD_THREADS, 1) k_wide(const __grid_constant__ 
                     for (int u = 0; u < 8; ++u) x[u] = ch * 8 + u < fin ? src[ch * 8 + u] : 0.0f;
                     uint32_t v[4];
                     pack8_16(x, v, f16);
-                    st_shared_v4(at + (uint32_t)ch * WD_XCOL, v[0], v[1], v[2], v[3]);
+                    st_shared_v4(at + (uint32_t)ch * xcol, v[0], v[1], v[2], v[3]);
                 }
                 __syncwarp();                              // the stage has been read
                 if (g + WD_LOADERS < groups)
@@ -366,11 +461,13 @@ __global__ void __launch_bounds__(WD_THREADS, 1) k_wide(const __grid_constant__ 
     } else {
         // ------------------------------------------------------ MMA issue
         const uint32_t id1 = idesc_16(WD_UNITS, n, f16), id2 = id1 | (1u << 16);
-        const uint32_t id3 = idesc_16(WD_ROWS, l3.N, f16) | (1u << 15);
-        const uint64_t xd = smem_desc(smem_u32(base + a.x), WD_XCOL, 128u);
-        const uint64_t h1d = smem_desc(smem_u32(base + a.h1), 1024u, 128u);
-        const uint64_t h2d = smem_desc(smem_u32(base + a.h2), 1024u, 128u);
-        const uint64_t w3d = smem_desc(smem_u32(base + a.w3), (uint32_t)(l3.N * 16), 128u);
+        const uint32_t id3 = idesc_16(WD_ROWS, WD_OUTS, f16) | (1u << 15);
+        // a K = 16 step of X or a hidden operand is two columns of n x 16 bytes
+        const uint32_t col = (uint32_t)(n * 16);
+        const uint64_t xd = smem_desc(smem_u32(base + a.x), col, 128u);
+        const uint64_t h1d = smem_desc(smem_u32(base + a.h1), col, 128u);
+        const uint64_t h2d = smem_desc(smem_u32(base + a.h2), col, 128u);
+        const uint64_t w3d = smem_desc(smem_u32(base + a.w3), (uint32_t)(WD_OUTS * 16), 128u);
         int m = 0;
         // tile t's first layer, tile t - 1's second, tile t - 2's third
         for (int t = 0; t < count + 2; ++t) {
@@ -382,8 +479,7 @@ __global__ void __launch_bounds__(WD_THREADS, 1) k_wide(const __grid_constant__ 
                 if (elect_one()) {
                     const uint64_t xb = xd + (uint64_t)(((uint32_t)b * a.x_bytes) >> 4);
                     for (int k = 0; k < ksteps1; ++k)
-                        mma_bf16_ta(tmem, w1t + 8u * (uint32_t)k, xb + (uint64_t)(2u * WD_XCOL / 16u * (uint32_t)k), id1,
-                                    k ? 1u : 0u);
+                        mma_bf16_ta(tmem, w1t + 8u * (uint32_t)k, xb + (uint64_t)(2 * n * k), id1, k ? 1u : 0u);
                     mma_commit(&bars->x_empty[b]);
                     mma_commit(&bars->a1_full);
                 }
@@ -396,9 +492,9 @@ __global__ void __launch_bounds__(WD_THREADS, 1) k_wide(const __grid_constant__ 
                 fence_proxy_async_smem();                  // the partner's half came by generic stores
                 tc_fence_after();
                 if (elect_one()) {
-                    const uint64_t hb = h1d + (uint64_t)(((uint32_t)b * WD_H) >> 4);
+                    const uint64_t hb = h1d + (uint64_t)(((uint32_t)b * a.h_bytes) >> 4);
                     for (int k = 0; k < ksteps2; ++k)
-                        mma_bf16_ta(tmem + WD_ACC2, w2t + 8u * (uint32_t)k, hb + (uint64_t)(128 * k), id2, k ? 1u : 0u);
+                        mma_bf16_ta(tmem + WD_ACC2, w2t + 8u * (uint32_t)k, hb + (uint64_t)(2 * n * k), id2, k ? 1u : 0u);
                     mma_commit(&bars->a2_full);
                 }
                 __syncwarp();
@@ -410,7 +506,8 @@ __global__ void __launch_bounds__(WD_THREADS, 1) k_wide(const __grid_constant__ 
                 tc_fence_after();
                 if (elect_one()) {
                     for (int k = 0; k < ksteps3; ++k)
-                        mma_bf16(tmem + WD_OUT, h2d + (uint64_t)(128 * k), w3d + (uint64_t)(2 * l3.N * k), id3, k ? 1u : 0u);
+                        mma_bf16(tmem + WD_OUT, h2d + (uint64_t)(2 * n * k), w3d + (uint64_t)(2 * WD_OUTS * k), id3,
+                                 k ? 1u : 0u);
                     mma_commit(&bars->o_full);
                 }
                 __syncwarp();
@@ -427,6 +524,8 @@ __global__ void __launch_bounds__(WD_THREADS, 1) k_wide(const __grid_constant__ 
             warp_wait_all(&bars->h1_full[i & 1], (uint32_t)(i >> 1) & 1u, true, &no_abort, a.err, 8u, TC_WAIT_NS);
         if (pair && owned > 0)
             warp_wait_all(&bars->h2_full, (uint32_t)(owned - 1) & 1u, true, &no_abort, a.err, 8u, TC_WAIT_NS);
+        if (a.act && agent == 0 && p.M > 1 && owned > 0)
+            warp_wait_all(&bars->comb_full, (uint32_t)(owned - 1) & 1u, true, &no_abort, a.err, 8u, TC_WAIT_NS);
     }
     __syncwarp();
     tc_fence_before();
@@ -437,10 +536,12 @@ __global__ void __launch_bounds__(WD_THREADS, 1) k_wide(const __grid_constant__ 
         tmem_dealloc(tmem, 512u);
     }
     __syncwarp();
-    if (pair) cluster_sync_all();                          // no peer touches this CTA's memory after it exits
+    if (size > 1) cluster_sync_all();                      // no peer touches this CTA's memory after it exits
 }
 
-// Shared memory of a launch (bytes, without the alignment slack).
+// Shared memory of a launch (bytes, without the alignment slack).  The hidden
+// operand of the output layer comes first: its M = 64 rows read past a shorter
+// tile's.
 uint32_t wd_layout(const TcPlan &p, WdArgs *a)
 {
     uint32_t off = 0;
@@ -449,22 +550,101 @@ uint32_t wd_layout(const TcPlan &p, WdArgs *a)
         off += (bytes + 127u) & ~127u;
         return at;
     };
-    const uint32_t x_bytes = (uint32_t)(p.layer[0].K / 8) * WD_XCOL;
-    const uint32_t stage_bytes = (uint32_t)(WD_GROUP * 4 * p.layer[0].fin);
-    const uint32_t h2 = take(WD_H), h1 = take(2u * WD_H), x = take(2u * x_bytes);
-    const uint32_t w3 = take((uint32_t)(p.layer[2].N * p.layer[2].K) * 2u), stage = take(WD_LOADERS * stage_bytes);
-    const uint32_t bars = take(sizeof(WdBars));
-    if (a) {
-        a->x_bytes = x_bytes;
-        a->stage_bytes = stage_bytes;
-        a->stage = stage;
-        a->h1 = h1;
-        a->h2 = h2;
-        a->x = x;
-        a->w3 = w3;
-        a->bars = bars;
-    }
+    a->x_bytes = (uint32_t)(p.layer[0].K / 8 * a->n * 16);
+    a->h_bytes = (uint32_t)(256 * a->n * 2);
+    a->stage_bytes = (uint32_t)(WD_GROUP * 4 * p.layer[0].fin);
+    a->h2 = take(a->h_bytes);
+    a->h1 = take(2u * a->h_bytes);
+    a->x = take(2u * a->x_bytes);
+    a->w3 = take((uint32_t)(WD_OUTS * p.layer[2].K) * 2u);
+    a->stage = take(WD_LOADERS * a->stage_bytes);
+    a->comb = a->act ? take((uint32_t)((p.M - 1) * a->n * WD_OUTS * 4)) : 0u;
+    a->bars = take(sizeof(WdBars));
     return off;
+}
+
+// Clusters of `size` CTAs the device holds at once (each CTA has an SM to
+// itself), queried once per device and size.
+int wd_clusters(int size, uint32_t smem, int device, int sms)
+{
+    static std::mutex mu;
+    static std::map<std::pair<int, int>, int> cache;
+    std::lock_guard<std::mutex> lk(mu);
+    const auto key = std::make_pair(device, size);
+    const auto it = cache.find(key);
+    if (it != cache.end()) return it->second;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(size * std::max(1, sms / size)), 1, 1);
+    cfg.blockDim = dim3(WD_THREADS, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)size;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, k_wide<WD_ROWS>, &cfg) != cudaSuccess || n < 1) {
+        cudaGetLastError();
+        n = std::max(1, sms / size);
+    }
+    n = std::min(n, std::max(1, sms / size));
+    cache[key] = n;
+    return n;
+}
+
+int wd_pair(const TcPlan &p) { return p.layer[0].N > WD_UNITS || p.layer[1].N > WD_UNITS ? 2 : 1; }
+
+// y: every agent's outputs, or (act) their weighted mean.
+int wd_launch(const fr_ensemble *e, const float *obs, int ld, int n, float *y, bool act, cudaStream_t s)
+{
+    const TcPlan &p = e->tc->plan;
+    WdArgs a;
+    memset(&a, 0, sizeof(a));
+    a.plan = p;
+    a.img = e->tc->img;
+    a.bias = e->tc->bias;
+    a.err = e->tc->err;
+    a.obs = obs;
+    a.ld = ld;
+    a.rows = n;
+    a.y = y;
+    a.act = act ? 1 : 0;
+    for (int j = 0; j < MAX_AGENTS; ++j) a.w[j] = e->host_weights[j];
+    a.nan0 = tc_small_batch(e, n);
+    a.bulk = ld == p.layer[0].fin && ((uintptr_t)obs & 15u) == 0;
+    a.pair = wd_pair(p);
+    const int size = a.pair * (act ? p.M : 1), most = act ? WD_ACT_ROWS : WD_ROWS;
+    a.n = most;
+    FR_CUDA(set_max_smem_once((const void *)k_wide<WD_ROWS>, e->ctx->device));
+    const int clusters = wd_clusters(size, wd_layout(p, &a) + 1024u, e->ctx->device, e->ctx->sm_count);
+    // tiles: as few rows each as spread the batch over every cluster in the
+    // waves it needs anyway
+    const int64_t lanes = std::max(1, act ? clusters : clusters / p.M);       // tiles in flight
+    const int64_t waves = (n + most * lanes - 1) / (most * lanes);
+    const int64_t per = (n + waves * lanes - 1) / (waves * lanes);
+    a.n = (int)std::min<int64_t>(most, (per + 15) / 16 * 16);
+    a.tiles = (int)ceil_div(n, a.n);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(size * (act ? 1 : p.M) * (int)std::min<int64_t>(lanes, a.tiles)), 1, 1);
+    cfg.blockDim = dim3(WD_THREADS, 1, 1);
+    cfg.dynamicSmemBytes = wd_layout(p, &a) + 1024u;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)size;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    // the weights load while the stream's previous kernel finishes
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    void (*const kern[4])(const WdArgs) = {k_wide<16>, k_wide<32>, k_wide<48>, k_wide<64>};
+    FR_CUDA(set_max_smem_once((const void *)kern[a.n / 16 - 1], e->ctx->device));
+    FR_CUDA(cudaLaunchKernelEx(&cfg, kern[a.n / 16 - 1], a));
+    return FR_OK;
 }
 
 }  // namespace
@@ -480,43 +660,21 @@ bool wd_ok(const fr_ensemble *e)
 
 int wd_forward(const fr_ensemble *e, const float *obs, int ld, int n, float *y, cudaStream_t s)
 {
-    const TcPlan &p = e->tc->plan;
-    WdArgs a;
-    memset(&a, 0, sizeof(a));
-    a.plan = p;
-    a.img = e->tc->img;
-    a.bias = e->tc->bias;
-    a.err = e->tc->err;
-    a.obs = obs;
-    a.ld = ld;
-    a.rows = n;
-    a.y = y;
-    a.nan0 = tc_small_batch(e, n);
-    a.bulk = ld == p.layer[0].fin && ((uintptr_t)obs & 15u) == 0;
-    a.pair = p.layer[0].N > WD_UNITS || p.layer[1].N > WD_UNITS ? 2 : 1;
-    const uint32_t smem = wd_layout(p, &a) + 1024u;
-    // tiles: as few rows each as spread the batch over every cluster in the
-    // waves it needs anyway
-    const int64_t per_agent = std::max(1, e->ctx->sm_count / a.pair / p.M);
-    const int64_t waves = (n + WD_ROWS * per_agent - 1) / (WD_ROWS * per_agent);
-    const int64_t per = (n + waves * per_agent - 1) / (waves * per_agent);
-    a.n = (int)std::min<int64_t>(WD_ROWS, (per + 15) / 16 * 16);
-    a.tiles = (int)ceil_div(n, a.n);
-    FR_CUDA(set_max_smem_once((const void *)k_wide, e->ctx->device));
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(a.pair * p.M * (int)std::min<int64_t>(per_agent, a.tiles)), 1, 1);
-    cfg.blockDim = dim3(WD_THREADS, 1, 1);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)a.pair;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    FR_CUDA(cudaLaunchKernelEx(&cfg, k_wide, a));
-    return FR_OK;
+    return wd_launch(e, obs, ld, n, y, false, s);
+}
+
+// Combining in the same launch: a cluster holds every agent (at most eight
+// CTAs).  23 clusters of six fit the GPU with 48 rows each, 25 pairs per agent
+// with 64: past four waves of the former a forward and a combining launch are
+// as fast.
+bool wd_act_ok(const fr_ensemble *e, int n)
+{
+    return wd_ok(e) && e->combine == FR_COMBINE_MEAN && wd_pair(e->tc->plan) * e->M <= 8 && n <= WD_ACT_MAX;
+}
+
+int wd_act(const fr_ensemble *e, const float *obs, int n, float *act, cudaStream_t s)
+{
+    return wd_launch(e, obs, e->dims[0], n, act, true, s);
 }
 
 }  // namespace fr

@@ -110,3 +110,25 @@ def test_narrow_rollout_equals_unfused(ctx, dev, N, M, hidden, auto_reset, prec)
         out.append({**tr, **st, "metrics": m})
     for k in out[0]:
         assert torch.equal(out[0][k], out[1][k]), k
+
+
+@pytest.mark.parametrize("dims,M", [((301, 256, 256, 30), 3), ((301, 256, 256, 30), 1), ((304, 255, 129, 32), 4),
+                                    ((61, 64, 64, 30), 5), ((61, 64, 64, 17), 2)])
+def test_act_equals_forward_then_mean(ctx, dev, dims, M):
+    # the agents combined in the forward's own launch, and (past its range) after it
+    w = np.random.default_rng(M).random(M).astype(np.float32)
+    ens = fr.ensemble_create(ctx, dims, synth.actor_params(dims, M, seed=M), weights=w, precision=fr.PREC_BF16)
+    wt = torch.from_numpy(w).to(dev)
+    n_max = 4500
+    x = torch.from_numpy(np.random.default_rng(3).standard_normal((n_max, dims[0])).astype(np.float32)).to(dev)
+    for n in (1, 8, 16, 17, 47, 48, 49, 1104, 1105, 1199, 2209, 4096, 4097, 4500):
+        y = torch.empty(M, n, dims[-1], device=dev)
+        act = torch.full((n + 1, dims[-1]), -7.0, device=dev)
+        fr.ensemble_forward(ens, x[:n].contiguous(), y)
+        fr.ensemble_act(ens, x[:n].contiguous(), act[:n])
+        want = y[0].clone()
+        for j in range(1, M):
+            want = want + wt[j] * (y[j] - y[0])
+        torch.cuda.synchronize()
+        assert torch.equal(act[:n], want) and (act[n] == -7.0).all()
+    assert fr.ensemble_device_errors(ens) == 0
