@@ -341,18 +341,44 @@ __device__ __noinline__ Fill own_buy_greedy(int64_t cash, int64_t want, int64_t 
     return Fill{cash, nb};
 }
 
-// fp32 trajectory observation of the step about to be taken (optional output,
-// out of line)
-__device__ __noinline__ void own_traj_obs(const F2Args &a, float *o, float cv, float pv, float hv, int day, int Ke,
-                                          int lane)
+// The trajectory-dependent entries of the fp32 trajectory observation of the
+// step about to be taken (optional output, out of line); k_traj_indicators
+// writes the others.
+__device__ __noinline__ void own_traj_obs(float *o, float cv, float pv, float hv, int lane)
 {
     if (lane == 0) o[0] = cv;
     if (lane < SK2) {
         o[1 + lane] = pv;
         o[1 + SK2 + lane] = hv;
     }
-    const float *f = a.v.ind + (int64_t)day * NIND;
-    for (int i = lane; i < NIND; i += 32) o[NSTATE + i] = (i % SK2) < Ke ? __ldg(f + i) : 0.0f;
+}
+
+// The 240 indicator entries of every row of a trajectory's observations.  The
+// day of (step, env) follows from the env's step count alone, so these leave
+// the rollout's step chain, where a row's 16 loads and stores were on the way
+// to the next step, for one pass over the output at memory speed (2,048 envs x
+// 64 steps: the rollout's kernel 626 -> 420 us, this pass 33 us).  Runs before
+// the rollout, which advances the counters.  A warp per row.
+__global__ void __launch_bounds__(256) k_traj_indicators(const EnvView v, int64_t rows, float *__restrict__ obs, int ld)
+{
+    const int64_t row = ((int64_t)blockIdx.x * 256 + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    if (row >= rows) return;
+    const int s = (int)(row / v.N), e = (int)(row - (int64_t)s * v.N);
+    const int t0 = v.t[e], W = v.W[e], Ke = v.Ke[e];
+    // done envs stand still, the others stop at (or restart before) day W - 1
+    const int t = v.done[e] ? t0 : (v.auto_reset ? (t0 + s) % (W - 1) : min(t0 + s, W - 1));
+    const float *f = v.ind + (int64_t)(v.start[e] + t) * NIND;
+    float *o = obs + row * ld + NSTATE;
+    float x[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+        const int i = lane + 32 * u;
+        x[u] = i < NIND && i % SK2 < Ke ? __ldg(f + i) : 0.0f;
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+        if (lane + 32 * u < NIND) o[lane + 32 * u] = x[u];
 }
 
 // The next observation row of env r: its 61 state entries in the A
@@ -469,8 +495,7 @@ __device__ __forceinline__ void own_publish_all(const F2Args &a, const OwnEnv *o
         for (int i = 0; i < NOWN; ++i) {
             const int e = eidx[i];
             if (e >= 0)
-                own_traj_obs(a, a.tr_obs + (tbase + e) * a.obs_ld, o[i].cv, o[i].pv, o[i].hv,
-                             own[i].start + own[i].t, own[i].Ke, lane);
+                own_traj_obs(a.tr_obs + (tbase + e) * a.obs_ld, o[i].cv, o[i].pv, o[i].hv, lane);
         }
     }
 }
@@ -1576,6 +1601,11 @@ int f2_rollout(fr_env *env, const fr_ensemble *e, int T, const fr_traj *traj, do
     // (a rollout in pieces is the same rollout).
     const int K = (!packed && !want_traj && !v.auto_reset && !env->split_off) ? std::min(F2_PIECES_MAX, T / 64) : 1;
     FR_CUDA(env_time_mark(env, 0, s));
+    if (traj->obs) {
+        const int64_t rows = (int64_t)T * v.N;
+        k_traj_indicators<<<ceil_div(rows * 32, 256), 256, 0, s>>>(v, rows, a.tr_obs, a.obs_ld);
+        FR_CUDA(cudaGetLastError());
+    }
     if (K <= 1) {
         FR_CUDA(cudaLaunchKernelEx(&cfg, kern, a));
         FR_CUDA(env_time_mark(env, 1, s));

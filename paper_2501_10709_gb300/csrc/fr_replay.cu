@@ -12,7 +12,7 @@
 // Push: the rows of a trajectory in (t, env) order; row (t, e) is a real
 // step unless the env was already done before it (done[t-1][e], or not live
 // at the start of the rollout), which frozen envs show without auto-reset.
-// Valid rows are appended in that order: a count kernel (one block per 1024
+// Valid rows are appended in that order: a count kernel (one block per 256
 // rows), a one-block scan that also advances the device counter, and a
 // scatter kernel that ranks its rows again and copies them, one warp per
 // row so that every copy is coalesced.  s' of row (t, e) is obs[t+1][e], or
@@ -28,7 +28,8 @@
 namespace fr {
 namespace {
 
-constexpr int RP_ROWS = 1024;         // rows per count / scatter block
+constexpr int RP_ROWS = 256;          // rows per count / scatter block (131,072 rows of 301: 131 us with 128
+                                      // blocks of 1,024 rows, 107 us with 512 of these)
 
 __device__ __forceinline__ bool rp_valid(int64_t r, int N, const uint8_t *done, const uint8_t *live0,
                                          int auto_reset)
@@ -129,7 +130,7 @@ __global__ void __launch_bounds__(RP_ROWS) k_rp_scatter(RpBuf b, int64_t rows, i
                                                         const int64_t *state)
 {
     __shared__ int64_t slot_s[RP_ROWS];
-    __shared__ int wcount[32];
+    __shared__ int wcount[RP_ROWS / 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t r0 = (int64_t)blockIdx.x * RP_ROWS;
     const int64_t r = r0 + threadIdx.x;
@@ -142,8 +143,8 @@ __global__ void __launch_bounds__(RP_ROWS) k_rp_scatter(RpBuf b, int64_t rows, i
     const int rank = before + __popc(m & ((1u << lane) - 1u));
     slot_s[threadIdx.x] = v ? (state[1] + offsets[blockIdx.x] + rank) % b.C : -1;
     __syncthreads();
-    // copy: warp w handles rows w, w + 32, ... of the block
-    for (int i = warp; i < RP_ROWS; i += 32) {
+    // copy: warp w handles rows w, w + 8, ... of the block
+    for (int i = warp; i < RP_ROWS; i += RP_ROWS / 32) {
         const int64_t slot = slot_s[i];
         if (slot < 0) continue;
         const int64_t row = r0 + i;
