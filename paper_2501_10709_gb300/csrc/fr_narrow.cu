@@ -280,6 +280,7 @@ __device__ __forceinline__ void nw_inputs(const NwArgs &a, NwBars *bars, const u
     const uint32_t at = smem_u32(base + a.sh.x) + (uint32_t)(i & 1) * (uint32_t)(NW_ROWS * 16) +
                         (uint32_t)(r / 8) * 128u + (uint32_t)(r % 8) * 16u;
     int k = 0;
+    grid_wait_previous();                        // whatever wrote the observations
     for (int tile = blockIdx.x; tile < a.tiles; tile += gridDim.x, ++k) {
         const int g = tile * n + r;
         const bool in = r < n && g < a.rows;
@@ -399,6 +400,7 @@ __global__ void __launch_bounds__(32 * (4 * NW_MAX_AGENTS + 4), 1) k_narrow(cons
         const int k2 = l2.K / 16, k3 = l3.K / 16;
         uint64_t *full = &bars->acc_full[j];
         uint32_t ph = 0;
+        if (!ROLL) grid_wait_previous();         // whatever still reads the outputs
         // no early exit: a wait that gives up sets the abort flag, the later
         // ones return after a poll, and the loop runs to its uniform end
         for (int s = 0; s < steps; ++s) {
@@ -516,8 +518,18 @@ int nw_launch(const fr_ensemble *e, const NwArgs &a, int grid, cudaStream_t s)
 {
     const uint32_t smem = a.sh.total + 1024u;
     FR_CUDA(set_max_smem_once((const void *)k_narrow<ROLL>, e->ctx->device));
-    k_narrow<ROLL><<<grid, 32 * (4 * a.sh.M + 4), smem, s>>>(a);
-    FR_CUDA(cudaGetLastError());
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid, 1, 1);
+    cfg.blockDim = dim3((unsigned)(32 * (4 * a.sh.M + 4)), 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    // a forward's weights load while the stream's previous kernel finishes
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = ROLL ? 0 : 1;
+    FR_CUDA(cudaLaunchKernelEx(&cfg, k_narrow<ROLL>, a));
     return FR_OK;
 }
 
