@@ -372,9 +372,11 @@ int tc_forward_tiled(const fr_ensemble *e, const float *obs, int ld, int n, floa
 // Narrow networks with every agent resident in one CTA (fr_narrow.cu): the
 // same results as tc_forward and the fused crypto rollout.
 bool nw_ok(const fr_ensemble *e);
+int nw_prepare(const fr_ensemble *e);
 int nw_forward(const fr_ensemble *e, const float *obs, int ld, int n, float *y, cudaStream_t s);
 // two hidden layers up to 256 wide, weights resident in CTA pairs (fr_wide.cu)
 bool wd_ok(const fr_ensemble *e);
+int wd_prepare(const fr_ensemble *e);
 int wd_forward(const fr_ensemble *e, const float *obs, int ld, int n, float *y, cudaStream_t s);
 // the weighted mean of the agents' outputs in the same launch, for batches wd_act_ok takes
 bool wd_act_ok(const fr_ensemble *e, int n);

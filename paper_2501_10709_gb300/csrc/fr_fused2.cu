@@ -1600,12 +1600,12 @@ int f2_rollout(fr_env *env, const fr_ensemble *e, int T, const fr_traj *traj, do
     // operation on `stream`.  Every env's arithmetic is that of one launch
     // (a rollout in pieces is the same rollout).
     const int K = (!packed && !want_traj && !v.auto_reset && !env->split_off) ? std::min(F2_PIECES_MAX, T / 64) : 1;
-    FR_CUDA(env_time_mark(env, 0, s));
     if (traj->obs) {
         const int64_t rows = (int64_t)T * v.N;
         k_traj_indicators<<<ceil_div(rows * 32, 256), 256, 0, s>>>(v, rows, a.tr_obs, a.obs_ld);
         FR_CUDA(cudaGetLastError());
     }
+    FR_CUDA(env_time_mark(env, 0, s));
     if (K <= 1) {
         FR_CUDA(cudaLaunchKernelEx(&cfg, kern, a));
         FR_CUDA(env_time_mark(env, 1, s));

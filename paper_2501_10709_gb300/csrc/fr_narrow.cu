@@ -545,6 +545,14 @@ bool nw_ok(const fr_ensemble *e)
            p.layer[1].K <= NW_UNITS && p.layer[2].K <= NW_UNITS;
 }
 
+// The kernel attributes of a forward, so that a first call may be inside a
+// stream capture.
+int nw_prepare(const fr_ensemble *e)
+{
+    FR_CUDA(set_max_smem_once((const void *)k_narrow<false>, e->ctx->device));
+    return FR_OK;
+}
+
 int nw_forward(const fr_ensemble *e, const float *obs, int ld, int n, float *y, cudaStream_t s)
 {
     NwArgs a;

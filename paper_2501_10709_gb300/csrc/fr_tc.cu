@@ -539,6 +539,8 @@ int tc_create(fr_ensemble *e)
         err = cudaFuncSetAttribute(k_tc_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
     e->tc = t;
     if (err != cudaSuccess) return cuda_fail(err, "tc_create upload");
+    if (nw_ok(e)) return nw_prepare(e);
+    if (wd_ok(e)) return wd_prepare(e);
     return FR_OK;
 }
 

@@ -45,7 +45,7 @@
 #include <cstring>
 #include <map>
 #include <mutex>
-#include <utility>
+#include <tuple>
 
 #include "fr_env_dev.cuh"
 #include "fr_ptx.cuh"
@@ -539,6 +539,8 @@ __global__ void __launch_bounds__(WD_THREADS, 1) k_wide(const __grid_constant__ 
     if (size > 1) cluster_sync_all();                      // no peer touches this CTA's memory after it exits
 }
 
+void (*const wd_kernels[4])(const WdArgs) = {k_wide<16>, k_wide<32>, k_wide<48>, k_wide<64>};   // by rows / 16
+
 // Shared memory of a launch (bytes, without the alignment slack).  The hidden
 // operand of the output layer comes first: its M = 64 rows read past a shorter
 // tile's.
@@ -564,13 +566,13 @@ uint32_t wd_layout(const TcPlan &p, WdArgs *a)
 }
 
 // Clusters of `size` CTAs the device holds at once (each CTA has an SM to
-// itself), queried once per device and size.
+// itself), queried once per device, size and shared memory.
 int wd_clusters(int size, uint32_t smem, int device, int sms)
 {
     static std::mutex mu;
-    static std::map<std::pair<int, int>, int> cache;
+    static std::map<std::tuple<int, int, uint32_t>, int> cache;
     std::lock_guard<std::mutex> lk(mu);
-    const auto key = std::make_pair(device, size);
+    const auto key = std::make_tuple(device, size, smem);
     const auto it = cache.find(key);
     if (it != cache.end()) return it->second;
     cudaLaunchConfig_t cfg = {};
@@ -641,9 +643,8 @@ int wd_launch(const fr_ensemble *e, const float *obs, int ld, int n, float *y, b
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    void (*const kern[4])(const WdArgs) = {k_wide<16>, k_wide<32>, k_wide<48>, k_wide<64>};
-    FR_CUDA(set_max_smem_once((const void *)kern[a.n / 16 - 1], e->ctx->device));
-    FR_CUDA(cudaLaunchKernelEx(&cfg, kern[a.n / 16 - 1], a));
+    FR_CUDA(set_max_smem_once((const void *)wd_kernels[a.n / 16 - 1], e->ctx->device));
+    FR_CUDA(cudaLaunchKernelEx(&cfg, wd_kernels[a.n / 16 - 1], a));
     return FR_OK;
 }
 
@@ -656,6 +657,24 @@ bool wd_ok(const fr_ensemble *e)
     const TcPlan &p = e->tc->plan;
     return p.esz == 2 && p.split == 1 && p.L == 3 && p.layer[0].K <= 304 && p.layer[0].N <= 256 &&
            p.layer[1].N <= 256 && p.layer[1].K <= 256 && p.layer[2].K <= 256 && p.layer[2].N <= 32;
+}
+
+// The host queries and kernel attributes of every launch shape, so that a
+// first call may be inside a stream capture.
+int wd_prepare(const fr_ensemble *e)
+{
+    WdArgs a;
+    memset(&a, 0, sizeof(a));
+    const TcPlan &p = e->tc->plan;
+    for (auto k : wd_kernels) FR_CUDA(set_max_smem_once((const void *)k, e->ctx->device));
+    a.n = WD_ROWS;
+    wd_clusters(wd_pair(p), wd_layout(p, &a) + 1024u, e->ctx->device, e->ctx->sm_count);
+    if (wd_act_ok(e, 1)) {
+        a.act = 1;
+        a.n = WD_ACT_ROWS;
+        wd_clusters(wd_pair(p) * p.M, wd_layout(p, &a) + 1024u, e->ctx->device, e->ctx->sm_count);
+    }
+    return FR_OK;
 }
 
 int wd_forward(const fr_ensemble *e, const float *obs, int ld, int n, float *y, cudaStream_t s)

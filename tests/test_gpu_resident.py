@@ -132,3 +132,27 @@ def test_act_equals_forward_then_mean(ctx, dev, dims, M):
         torch.cuda.synchronize()
         assert torch.equal(act[:n], want) and (act[n] == -7.0).all()
     assert fr.ensemble_device_errors(ens) == 0
+
+
+@pytest.mark.parametrize("dims,M,combine", [((301, 256, 256, 30), 3, "mean"), ((10, 128, 128, 3), 5, "vote")])
+def test_first_call_inside_a_capture(ctx, dev, dims, M, combine):
+    # a new ensemble's first forward and act, captured; replays equal direct calls on other inputs
+    vote = combine == "vote"
+    ens = fr.ensemble_create(ctx, dims, synth.actor_params(dims, M, seed=9), precision=fr.PREC_FP16,
+                             combine=fr.COMBINE_VOTE if vote else fr.COMBINE_MEAN, out_act=0 if vote else 1)
+    n = 70
+    x, y = torch.zeros(n, dims[0], device=dev), torch.empty(M, n, dims[-1], device=dev)
+    a = torch.empty(n, dtype=torch.uint8, device=dev) if vote else torch.empty(n, dims[-1], device=dev)
+    torch.cuda.synchronize()
+    g, side = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    with torch.cuda.graph(g, stream=side):
+        fr.ensemble_forward(ens, x, y, stream=side)
+        fr.ensemble_act(ens, x, a, stream=side)
+    for seed in range(3):
+        x.copy_(torch.from_numpy(np.random.default_rng(seed).standard_normal((n, dims[0])).astype(np.float32)))
+        g.replay()
+        y2, a2 = torch.empty_like(y), torch.empty_like(a)
+        fr.ensemble_forward(ens, x, y2)
+        fr.ensemble_act(ens, x, a2)
+        torch.cuda.synchronize()
+        assert torch.equal(y, y2) and torch.equal(a, a2)
