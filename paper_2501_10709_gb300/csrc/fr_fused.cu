@@ -1017,7 +1017,8 @@ int tc_rollout(fr_env *env, const fr_ensemble *e, int T, const fr_traj *traj, do
         return FR_OK;
     }
     // value log [T][N] in the env's scratch (grown outside any timed region)
-    const uint64_t need = (uint64_t)T * v.N * 8;
+    const bool narrow = v.task == FR_TASK_CRYPTO && nw_ok(e) && !ring;
+    const uint64_t need = narrow ? nw_rollout_scratch(env, T) : (uint64_t)T * v.N * 8;
     if (env->scratch_bytes < need) {
         FR_CUDA(cudaStreamSynchronize(s));
         dev_free(env->ctx, env->scratch, env->scratch_bytes);
@@ -1027,13 +1028,8 @@ int tc_rollout(fr_env *env, const fr_ensemble *e, int T, const fr_traj *traj, do
         if (rc) return rc;
         env->scratch_bytes = need;
     }
-    if (v.task == FR_TASK_CRYPTO && nw_ok(e) && !ring) {
-        FR_CUDA(env_time_mark(env, 0, s));
-        const int rc = nw_rollout(env, e, T, traj, (int64_t *)env->scratch, s);
-        if (rc) return rc;
-        FR_CUDA(env_time_mark(env, 1, s));
-        FR_CUDA(launch_metrics_replay(v, (const int64_t *)env->scratch, T, metrics, s));
-        return FR_OK;
+    if (narrow) {
+        return nw_rollout(env, e, T, traj, env->scratch, metrics, s);
     }
     FusedArgs a;
     memset(&a, 0, sizeof(a));

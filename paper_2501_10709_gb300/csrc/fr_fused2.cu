@@ -208,7 +208,6 @@ __host__ __device__ inline F2Smem f2_smem(const F2Plan &p)
 }
 
 // pieces of a split rollout (launches of the resident kernel per rollout)
-constexpr int F2_PIECES_MAX = 4;
 
 // barrier slots
 enum { B_W = 0, B_OBS, B_ACC, B_H1, B_H2, B_X, B_END, B_COUNT };
@@ -1458,7 +1457,7 @@ int f2_rollout(fr_env *env, const fr_ensemble *e, int T, const fr_traj *traj, do
     }
     // the value log, then one [N] array of start step counts per launch
     const uint64_t t0_b = ((uint64_t)v.N * 4 + 255) & ~255ull;
-    const uint64_t vlog_b = (((uint64_t)T * v.N * 8 + 255) & ~255ull) + (uint64_t)F2_PIECES_MAX * t0_b;
+    const uint64_t vlog_b = (((uint64_t)T * v.N * 8 + 255) & ~255ull) + (uint64_t)SPLIT_PIECES_MAX * t0_b;
     if (env->scratch_bytes < vlog_b) {
         FR_CUDA(cudaStreamSynchronize(s));
         dev_free(env->ctx, env->scratch, env->scratch_bytes);
@@ -1599,7 +1598,7 @@ int f2_rollout(fr_env *env, const fr_ensemble *e, int T, const fr_traj *traj, do
     // two streams, so the rollout stays one ordered (and graph-capturable)
     // operation on `stream`.  Every env's arithmetic is that of one launch
     // (a rollout in pieces is the same rollout).
-    const int K = (!packed && !want_traj && !v.auto_reset && !env->split_off) ? std::min(F2_PIECES_MAX, T / 64) : 1;
+    const int K = (!packed && !want_traj && !v.auto_reset && !env->split_off) ? std::min(SPLIT_PIECES_MAX, T / 64) : 1;
     if (traj->obs) {
         const int64_t rows = (int64_t)T * v.N;
         k_traj_indicators<<<ceil_div(rows * 32, 256), 256, 0, s>>>(v, rows, a.tr_obs, a.obs_ld);
@@ -1612,59 +1611,23 @@ int f2_rollout(fr_env *env, const fr_ensemble *e, int T, const fr_traj *traj, do
         FR_CUDA(launch_metrics_replay(v, vlog, T, metrics, s, t0a));
         return FR_OK;
     }
-    if (!env->split_stream) {
-        int lo = 0, hi = 0;
-        FR_CUDA(cudaDeviceGetStreamPriorityRange(&lo, &hi));
-        FR_CUDA(cudaStreamCreateWithPriority(&env->split_stream, cudaStreamNonBlocking, hi));
-        for (int i = 0; i <= F2_PIECES_MAX; ++i)
-            FR_CUDA(cudaEventCreateWithFlags(&env->split_ev[i], cudaEventDisableTiming));
-        env->split_prio = hi;
-    }
-    cudaLaunchConfig_t cfg2 = cfg;
-    cudaLaunchAttribute attr2[2];
-    attr2[0] = attr[0];
-    attr2[1].id = cudaLaunchAttributePriority;
-    attr2[1].val.priority = env->split_prio;
-    cfg2.attrs = attr2;
-    cfg2.numAttrs = 2;
-    cfg2.stream = env->split_stream;
-    FR_CUDA(cudaEventRecord(env->split_ev[F2_PIECES_MAX], s));
-    FR_CUDA(cudaStreamWaitEvent(env->split_stream, env->split_ev[F2_PIECES_MAX], 0));
-    // the pieces' ends: the last piece is short (T / 8), so that the replay
-    // left after the kernel is short, the one before it T / 4, and the
-    // others share the rest evenly (80, 80, 64 and 32 steps at T = 256;
-    // measured 1.720 ms per rollout against 1.747 with 74, 75, 75 and 32)
-    int ends[F2_PIECES_MAX];
-    {
-        const int tl = std::max(16, T / 8), tp = std::max(16, T / 4);
-        const int head = K >= 3 ? T - tl - tp : T - tl;        // the evenly shared steps
-        const int nh = K >= 3 ? K - 2 : K - 1;                 // pieces sharing them
-        for (int k = 0; k < nh; ++k) ends[k] = (k + 1) * head / nh;
-        if (K >= 3) ends[K - 2] = T - tl;
-        ends[K - 1] = T;
-    }
-    int s0 = 0;
-    for (int k = 0; k < K; ++k) {
-        const int Tk = ends[k] - s0;
-        F2Args b = a;
-        b.T = Tk;
-        b.vlog = vlog + (int64_t)s0 * v.N;
-        b.t0_out = (int32_t *)((char *)t0a + (uint64_t)k * t0_b);
-        b.ex.g0 = a.ex.g0 + (uint32_t)s0;
-        FR_CUDA(cudaLaunchKernelEx(&cfg2, kern, b));               // steps [s0, s0 + Tk)
-        FR_CUDA(cudaEventRecord(env->split_ev[k], env->split_stream));
-        s0 += Tk;
-    }
-    s0 = 0;
-    for (int k = 0; k < K; ++k) {
-        const int Tk = ends[k] - s0;
-        FR_CUDA(cudaStreamWaitEvent(s, env->split_ev[k], 0));
-        if (k == K - 1) FR_CUDA(env_time_mark(env, 1, s));
-        FR_CUDA(launch_metrics_replay(v, vlog + (int64_t)s0 * v.N, Tk, k == K - 1 ? metrics : nullptr, s,
-                                      (const int32_t *)((const char *)t0a + (uint64_t)k * t0_b)));
-        s0 += Tk;
-    }
-    return FR_OK;
+    return split_rollout(env, T, K, vlog, t0a, t0_b, metrics, s,
+                         [&](int s0, int Tk, int64_t *log, int32_t *t0, cudaStream_t ks, int prio) {
+                             cudaLaunchConfig_t cfg2 = cfg;
+                             cudaLaunchAttribute attr2[2];
+                             attr2[0] = attr[0];
+                             attr2[1].id = cudaLaunchAttributePriority;
+                             attr2[1].val.priority = prio;
+                             cfg2.attrs = attr2;
+                             cfg2.numAttrs = 2;
+                             cfg2.stream = ks;
+                             F2Args b = a;
+                             b.T = Tk;
+                             b.vlog = log;
+                             b.t0_out = t0;
+                             b.ex.g0 = a.ex.g0 + (uint32_t)s0;
+                             return cudaLaunchKernelEx(&cfg2, kern, b);
+                         });
 }
 
 }  // namespace fr

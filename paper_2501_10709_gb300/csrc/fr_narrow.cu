@@ -28,9 +28,9 @@
 // last MMA and the next operand there is only argmax, vote and a select.
 //
 // Measured: the 8,192-env, 1,024-step crypto rollout of five 10-128-128-3
-// networks 16.4 -> 3.6 ms (13.4 -> 3.1 us per step with one CTA per agent and
-// 128-row tile before; 0.44 ms of it is the value log's replay); Q targets of
-// 65,536 rows, two such forwards, 170 -> 58 us.  A step is a chain of three MMA
+// networks 16.4 -> 3.3 ms (a step 13.4 -> 3.1 us with one CTA per agent and
+// 128-row tile before); Q targets of 65,536 rows, two such forwards, 170 -> 50
+// us.  A step is a chain of three MMA
 // round trips, two epilogues and the vote (about 5,900 cycles); its 85 MMAs
 // take the tensor pipe 2,700 of them (32 to 47 cycles per K = 16 step of 64
 // rows with the weights in tensor or shared memory, 24 in the output layer).
@@ -79,6 +79,7 @@ struct NwArgs {
     float *tr_rew_f32;
     uint8_t *tr_done;
     int64_t *vlog;                               // [T][N]
+    int32_t *t0_out;                             // [N] step counts at the start, the env's then advanced; or NULL
     Explore ex;
 };
 
@@ -149,6 +150,7 @@ __device__ __forceinline__ void nw_env(const NwArgs &a, NwBars *bars, const uint
         start = v.start[e];
         W = v.W[e];
         pos = v.hold[e];
+        if (a.t0_out) a.t0_out[e] = t;
     }
     auto word0 = [&](int64_t c, int p) {
         return pack2_16(obs_scale(c, 1e-8f), __fdiv_rn(__int2float_rn(p), __int2float_rn(v.pmax)), f16);
@@ -260,8 +262,9 @@ __device__ __forceinline__ void nw_env(const NwArgs &a, NwBars *bars, const uint
         }
         __syncwarp();
     }
-    // steps and accumulators follow from the value log
+    // steps (unless recorded) and accumulators follow from the value log
     if (e >= 0) {
+        if (a.t0_out) v.t[e] = t;
         v.cash[e] = cash;
         v.done[e] = done ? 1 : 0;
         v.hold[e] = pos;
@@ -513,26 +516,6 @@ int nw_tile_rows(int64_t n, int sms)
     return (int)std::min<int64_t>(NW_ROWS, (std::max<int64_t>(per, 1) + 15) / 16 * 16);
 }
 
-template <bool ROLL>
-int nw_launch(const fr_ensemble *e, const NwArgs &a, int grid, cudaStream_t s)
-{
-    const uint32_t smem = a.sh.total + 1024u;
-    FR_CUDA(set_max_smem_once((const void *)k_narrow<ROLL>, e->ctx->device));
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)grid, 1, 1);
-    cfg.blockDim = dim3((unsigned)(32 * (4 * a.sh.M + 4)), 1, 1);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    // a forward's weights load while the stream's previous kernel finishes
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = ROLL ? 0 : 1;
-    FR_CUDA(cudaLaunchKernelEx(&cfg, k_narrow<ROLL>, a));
-    return FR_OK;
-}
-
 }  // namespace
 
 // Networks k_narrow takes.
@@ -568,11 +551,33 @@ int nw_forward(const fr_ensemble *e, const float *obs, int ld, int n, float *y, 
     a.nan0 = tc_small_batch(e, n);
     a.tiles = (int)ceil_div(n, a.sh.n);
     a.y = y;
-    return nw_launch<false>(e, a, std::min(a.tiles, std::max(1, e->ctx->sm_count)), s);
+    FR_CUDA(set_max_smem_once((const void *)k_narrow<false>, e->ctx->device));
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)std::min(a.tiles, std::max(1, e->ctx->sm_count)), 1, 1);
+    cfg.blockDim = dim3((unsigned)(32 * (4 * a.sh.M + 4)), 1, 1);
+    cfg.dynamicSmemBytes = a.sh.total + 1024u;
+    cfg.stream = s;
+    // the weights load while the stream's previous kernel finishes
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    FR_CUDA(cudaLaunchKernelEx(&cfg, k_narrow<false>, a));
+    return FR_OK;
 }
 
-// The crypto rollout's launch; vlog [T][N].
-int nw_rollout(fr_env *env, const fr_ensemble *e, int T, const fr_traj *traj, int64_t *vlog, cudaStream_t s)
+uint64_t nw_rollout_scratch(const fr_env *env, int T)
+{
+    const uint64_t log = ((uint64_t)T * env->v.N * 8 + 255) & ~255ull, t0 = (4ull * env->v.N + 255) & ~255ull;
+    return log + SPLIT_PIECES_MAX * t0;
+}
+
+// The crypto rollout: one launch and the replay of its value log, or, where
+// the tiles leave SMs idle (8,192 envs: 24 of 152), in pieces whose replays
+// run there (3.59 -> 3.31 ms for 1,024 steps).
+int nw_rollout(fr_env *env, const fr_ensemble *e, int T, const fr_traj *traj, void *scratch, double *metrics,
+               cudaStream_t s)
 {
     const EnvView &v = env->v;
     NwArgs a;
@@ -590,9 +595,44 @@ int nw_rollout(fr_env *env, const fr_ensemble *e, int T, const fr_traj *traj, in
     a.tr_rew = traj->rew;
     a.tr_rew_f32 = traj->rew_f32;
     a.tr_done = traj->done;
-    a.vlog = vlog;
+    a.vlog = (int64_t *)scratch;
     a.ex = explore_of(env, env->explore_step);
-    return nw_launch<true>(e, a, (int)ceil_div(v.N, a.sh.n), s);
+    const int grid = (int)ceil_div(v.N, a.sh.n);
+    const bool want_traj = traj->obs || traj->act || traj->rew || traj->rew_f32 || traj->done;
+    const int K = !want_traj && !v.auto_reset && !env->split_off && grid < env->ctx->sm_count
+                      ? std::min(SPLIT_PIECES_MAX, T / 64)
+                      : 1;
+    FR_CUDA(set_max_smem_once((const void *)k_narrow<true>, env->ctx->device));
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid, 1, 1);
+    cfg.blockDim = dim3((unsigned)(32 * (4 * a.sh.M + 4)), 1, 1);
+    cfg.dynamicSmemBytes = a.sh.total + 1024u;
+    cfg.stream = s;
+    FR_CUDA(env_time_mark(env, 0, s));
+    if (K <= 1) {
+        FR_CUDA(cudaLaunchKernelEx(&cfg, k_narrow<true>, a));
+        FR_CUDA(env_time_mark(env, 1, s));
+        FR_CUDA(launch_metrics_replay(v, a.vlog, T, metrics, s));
+        return FR_OK;
+    }
+    const uint64_t t0_b = (4ull * v.N + 255) & ~255ull;
+    int32_t *t0a = (int32_t *)((char *)scratch + (((uint64_t)T * v.N * 8 + 255) & ~255ull));
+    return split_rollout(env, T, K, a.vlog, t0a, t0_b, metrics, s,
+                         [&](int s0, int Tk, int64_t *log, int32_t *t0, cudaStream_t ks, int prio) {
+                             cudaLaunchAttribute attr[1];
+                             attr[0].id = cudaLaunchAttributePriority;
+                             attr[0].val.priority = prio;
+                             cudaLaunchConfig_t c = cfg;
+                             c.attrs = attr;
+                             c.numAttrs = 1;
+                             c.stream = ks;
+                             NwArgs b = a;
+                             b.T = Tk;
+                             b.vlog = log;
+                             b.t0_out = t0;
+                             b.ex.g0 = a.ex.g0 + (uint32_t)s0;
+                             return cudaLaunchKernelEx(&c, k_narrow<true>, b);
+                         });
 }
 
 }  // namespace fr

@@ -156,3 +156,48 @@ def test_first_call_inside_a_capture(ctx, dev, dims, M, combine):
         fr.ensemble_act(ens, x, a2)
         torch.cuda.synchronize()
         assert torch.equal(y, y2) and torch.equal(a, a2)
+
+
+@pytest.mark.parametrize("explore", [False, True])
+def test_narrow_rollout_in_pieces(ctx, dev, explore):
+    # 200 steps in three pieces whose replays run beside the next, then 130 in
+    # two, equal single launches; and a captured rollout replays them
+    N = 700
+    mk = fr.fr_market_create(ctx, synth.crypto_market(30_000, seed=6))
+    e = synth.crypto_envs(N, 30_000, 500, seed=6)
+    W = np.random.default_rng(6).integers(2, 400, N).astype(np.int32)
+    ens = fr.ensemble_create(ctx, (10, 64, 128, 3), synth.actor_params((10, 64, 128, 3), 5, seed=6, out_scale=4.0),
+                             precision=fr.PREC_FP16, combine=fr.COMBINE_VOTE, out_act=0)
+
+    def run(env, lengths):
+        out = []
+        for T in lengths:
+            m = torch.empty(N, 3, dtype=torch.float64, device=dev)
+            fr.rollout(env, ens, T, metrics=m)
+            st = [torch.empty(N, dtype=t, device=dev) for t in (torch.int64, torch.int32, torch.int32, torch.uint8)]
+            fr.env_get_state(env, cash=st[0], hold=st[1], steps=st[2], done=st[3])
+            out += [m] + st
+        return out
+
+    envs = []
+    for split in (False, True):
+        env = fr.env_create(ctx, mk, start=e.start, window=W, pmax=3)
+        fr.env_set_rollout_split(env, split)
+        if explore:
+            fr.env_set_exploration(env, fr.EXPLORE_EPS_GREEDY, eps=0.3, seed=5)
+        envs.append(env)
+    a, b = run(envs[0], (200, 130)), run(envs[1], (200, 130))
+    torch.cuda.synchronize()
+    assert all(torch.equal(x, y) for x, y in zip(a, b))
+    if explore:
+        return
+    g, side = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    m = torch.empty(N, 3, dtype=torch.float64, device=dev)
+    with torch.cuda.graph(g, stream=side):
+        fr.env_reset(envs[1], stream=side)
+        fr.rollout(envs[1], ens, 200, metrics=m, stream=side)
+    for _ in range(2):
+        m.fill_(-7.0)
+        g.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(m, a[0])
