@@ -512,10 +512,10 @@ int env_tile_packing_efficiency(const fr_env *env, float *eff);
  * are captured with the rollout into a graph).  No counterpart in the paper. */
 int env_set_table_cache(fr_env *env, int32_t on);
 
-/* Split fused stock rollouts (no counterpart in the paper).  on = 1 (the
- * default): a fused stock rollout of T >= 128 steps, without tile packing,
- * trajectory outputs or auto-reset, runs as K = min(4, T / 64) launches of
- * the resident kernel (the last T / 8 steps, the one before it T / 4, the
+/* Split fused rollouts (no counterpart in the paper).  on = 1 (the default):
+ * a fused stock rollout, or a BF16 / FP16 crypto rollout whose tiles leave
+ * SMs idle, of T >= 128 steps, without tile packing, trajectory outputs or
+ * auto-reset, runs as K = min(4, T / 64) launches of the resident kernel (the last T / 8 steps, the one before it T / 4, the
  * others sharing the rest evenly) on an internal stream of the highest
  * priority, and the FP64 metrics replay of each piece runs on `stream`
  * beside the next piece, so that only the last piece's replay follows the
