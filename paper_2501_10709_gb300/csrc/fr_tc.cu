@@ -526,7 +526,7 @@ int tc_create(fr_ensemble *e)
     if (err == cudaSuccess && grouped) err = cudaMemcpy(t->img2, img2.data(), ib, cudaMemcpyHostToDevice);
     if (err == cudaSuccess) err = cudaMemcpy(t->bias, bias.data(), bb, cudaMemcpyHostToDevice);
     if (err == cudaSuccess) err = cudaMemset(t->err, 0, 256);
-    int optin = 0;
+    int &optin = t->optin;
     if (err == cudaSuccess)
         err = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, e->ctx->device);
     if (err == cudaSuccess && tc_smem_bytes(p) > (uint32_t)optin) {

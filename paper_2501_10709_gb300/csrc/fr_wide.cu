@@ -565,8 +565,21 @@ uint32_t wd_layout(const TcPlan &p, WdArgs *a)
     return off;
 }
 
+// Rows of the tallest tile: 48 where the agents are combined, else 64, or fewer
+// where the operands of 64 do not fit the SM (inputs of 303 or 304 before a
+// second hidden layer wider than 240 take 48).
+int wd_most(const TcPlan &p, bool act, int optin)
+{
+    WdArgs a;
+    memset(&a, 0, sizeof(a));
+    a.act = act ? 1 : 0;
+    for (a.n = act ? WD_ACT_ROWS : WD_ROWS; a.n > 16 && wd_layout(p, &a) + 1024u > (uint32_t)optin;) a.n -= 16;
+    return a.n;
+}
+
 // Clusters of `size` CTAs the device holds at once (each CTA has an SM to
-// itself), queried once per device, size and shared memory.
+// itself), queried once per device, size and shared memory; 0 when it holds
+// none or the query fails.
 int wd_clusters(int size, uint32_t smem, int device, int sms)
 {
     static std::mutex mu;
@@ -589,7 +602,7 @@ int wd_clusters(int size, uint32_t smem, int device, int sms)
     int n = 0;
     if (cudaOccupancyMaxActiveClusters(&n, k_wide<WD_ROWS>, &cfg) != cudaSuccess || n < 1) {
         cudaGetLastError();
-        n = std::max(1, sms / size);
+        return 0;
     }
     n = std::min(n, std::max(1, sms / size));
     cache[key] = n;
@@ -617,10 +630,12 @@ int wd_launch(const fr_ensemble *e, const float *obs, int ld, int n, float *y, b
     a.nan0 = tc_small_batch(e, n);
     a.bulk = ld == p.layer[0].fin && ((uintptr_t)obs & 15u) == 0;
     a.pair = wd_pair(p);
-    const int size = a.pair * (act ? p.M : 1), most = act ? WD_ACT_ROWS : WD_ROWS;
+    const int size = a.pair * (act ? p.M : 1), most = wd_most(p, act, e->tc->optin);
     a.n = most;
     FR_CUDA(set_max_smem_once((const void *)k_wide<WD_ROWS>, e->ctx->device));
     const int clusters = wd_clusters(size, wd_layout(p, &a) + 1024u, e->ctx->device, e->ctx->sm_count);
+    FR_CHECK(clusters > 0, FR_ECUDA, "no room for clusters of %d CTAs with %u bytes of shared memory each", size,
+             wd_layout(p, &a) + 1024u);
     // tiles: as few rows each as spread the batch over every cluster in the
     // waves it needs anyway
     const int64_t lanes = std::max(1, act ? clusters : clusters / p.M);       // tiles in flight
@@ -667,11 +682,11 @@ int wd_prepare(const fr_ensemble *e)
     memset(&a, 0, sizeof(a));
     const TcPlan &p = e->tc->plan;
     for (auto k : wd_kernels) FR_CUDA(set_max_smem_once((const void *)k, e->ctx->device));
-    a.n = WD_ROWS;
+    a.n = wd_most(p, false, e->tc->optin);
     wd_clusters(wd_pair(p), wd_layout(p, &a) + 1024u, e->ctx->device, e->ctx->sm_count);
     if (wd_act_ok(e, 1)) {
         a.act = 1;
-        a.n = WD_ACT_ROWS;
+        a.n = wd_most(p, true, e->tc->optin);
         wd_clusters(wd_pair(p) * p.M, wd_layout(p, &a) + 1024u, e->ctx->device, e->ctx->sm_count);
     }
     return FR_OK;
