@@ -77,7 +77,7 @@ struct WdArgs {
     float *y;
     int pair, n, tiles, nan0;                     // CTAs per agent, rows per tile, tiles of the batch
     int act;                                      // 1: y is the weighted mean of the agents [rows][outputs]
-    float w[MAX_AGENTS];
+    const float *w;                               // the agents' weights (device), read by every launch and replay
     uint32_t x_bytes, h_bytes, stage_bytes, w3, x, h1, h2, stage, comb, bars;   // shared memory
     int bulk;                                     // rows are packed and 16-byte aligned: bulk copies
 };
@@ -93,6 +93,7 @@ struct WdBars {
     uint64_t drain;
     uint32_t tmem;
     int abort;
+    float w[4][MAX_AGENTS];                       // combine weights, a copy per output warp
 };
 
 __device__ __forceinline__ void wd_wait(uint64_t *bar, uint32_t parity, bool remote, volatile int *abort,
@@ -194,6 +195,7 @@ __device__ __forceinline__ void wd_combine(const WdArgs &a, WdBars *bars, uint8_
     const int fout = p.layer[2].fout, lane = threadIdx.x & 31;
     volatile int *abort = &bars->abort;
     const uint32_t comb = smem_u32(base + a.comb);
+    const float *w = bars->w[(threadIdx.x >> 5) & 3];
     uint32_t far = 0u, far_bar = 0u;
     if (agent > 0) {
         far = map_shared_rank(comb, (uint32_t)c) + (uint32_t)(((agent - 1) * n + r) * 128);
@@ -222,7 +224,7 @@ __device__ __forceinline__ void wd_combine(const WdArgs &a, WdBars *bars, uint8_
                 const uint32_t ou[4] = {o.x, o.y, o.z, o.w};
 #pragma unroll
                 for (int u = 0; u < 4; ++u)
-                    acc[u] = __fadd_rn(acc[u], __fmul_rn(a.w[j], __fsub_rn(__uint_as_float(ou[u]), x[u])));
+                    acc[u] = __fadd_rn(acc[u], __fmul_rn(w[j], __fsub_rn(__uint_as_float(ou[u]), x[u])));
             }
 #pragma unroll
             for (int u = 0; u < 4; ++u)
@@ -384,6 +386,10 @@ __global__ void __launch_bounds__(WD_THREADS, 1) k_wide(const __grid_constant__ 
         const float *b3 = a.bias + ((size_t)agent * MAX_LAYERS + 2) * 256;
         const float bl = lane < l3.N ? b3[lane] : 0.0f;
         grid_wait_previous();                              // whatever still reads the outputs
+        if (a.act) {
+            if (lane < p.M) bars->w[q][lane] = a.w[lane];
+            __syncwarp();
+        }
         for (int m = 0; m < owned; ++m) {
             const int i = pair ? 2 * m + c : m;
             if (n <= WD_ACT_ROWS && a.act && agent == 0 && p.M > 1 && q == 0 && lane == 0)
@@ -626,7 +632,7 @@ int wd_launch(const fr_ensemble *e, const float *obs, int ld, int n, float *y, b
     a.rows = n;
     a.y = y;
     a.act = act ? 1 : 0;
-    for (int j = 0; j < MAX_AGENTS; ++j) a.w[j] = e->host_weights[j];
+    a.w = e->weights;
     a.nan0 = tc_small_batch(e, n);
     a.bulk = ld == p.layer[0].fin && ((uintptr_t)obs & 15u) == 0;
     a.pair = wd_pair(p);

@@ -40,3 +40,26 @@ def test_shapes_at_the_shared_memory_limit(ctx, dev, dims, prec):
         assert torch.equal(y, full[:, :n])
         assert torch.equal(act, y[0] + w * (y[1] - y[0]) + w * (y[2] - y[0]))
     assert fr.ensemble_device_errors(ens) == 0
+
+
+@pytest.mark.parametrize("prec", [fr.PREC_BF16, fr.PREC_FP32])
+@pytest.mark.parametrize("n", [8, 1500, 4500])
+def test_captured_act_follows_new_weights(ctx, dev, n, prec):
+    # a replayed act uses the weights set since its capture, at every batch size
+    dims, M = (61, 64, 200, 30), 3
+    ens = fr.ensemble_create(ctx, dims, synth.actor_params(dims, M, seed=2), precision=prec)
+    x = torch.from_numpy(np.random.default_rng(2).standard_normal((n, dims[0])).astype(np.float32)).to(dev)
+    a, b = torch.empty(n, dims[-1], device=dev), torch.empty(n, dims[-1], device=dev)
+    torch.cuda.synchronize()
+    g, side = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    with torch.cuda.graph(g, stream=side):
+        fr.ensemble_act(ens, x, a, stream=side)
+    seen = []
+    for w in ((0.2, 0.3, 0.5), (0.0, 1.0, 0.0), (0.1, 0.0, 0.9)):
+        fr.ensemble_set_weights(ens, np.float32(w))
+        g.replay()
+        fr.ensemble_act(ens, x, b)
+        torch.cuda.synchronize()
+        assert torch.equal(a, b)
+        seen.append(a.clone())
+    assert not torch.equal(seen[0], seen[1]) and not torch.equal(seen[1], seen[2])
