@@ -193,7 +193,7 @@ int forward_any(const fr_ensemble *e, const float *obs, int ld, int n, float *y,
 {
     if (e->precision != FR_PREC_FP32) {
         const uint64_t tb = tc_tiled_scratch_bytes(e, n);
-        if (tb == 0) return tc_forward(e, obs, ld, n, y, s);
+        if (tb == 0) return tc_forward(e, obs, ld, n, y, s, true);
         void *tiles = nullptr;
         FR_CUDA(cudaMallocAsync(&tiles, tb, s));
         const int rc = tc_forward_tiled(e, obs, ld, n, y, tiles, s);
@@ -1118,7 +1118,7 @@ static int plain_rollout(fr_env *env, const fr_ensemble *e, int32_t T, const fr_
             FR_CUDA(forward_plain(e, obs_t, ldt, N, y, hid, s));
         } else {
             rc = tiles ? tc_forward_tiled(e, obs_t, ldt, N, y, tiles, s) : FR_EINVAL;
-            if (rc == FR_EINVAL) rc = tc_forward(e, obs_t, ldt, N, y, s);
+            if (rc == FR_EINVAL) rc = tc_forward(e, obs_t, ldt, N, y, s, tiled_ok);
             if (rc) return rc;
         }
         void *act_t = traj->act ? (stock ? (void *)((float *)traj->act + row * v.K)

@@ -360,7 +360,9 @@ cudaError_t forward_plain(const fr_ensemble *e, const float *obs, int ld, int n,
 int tc_create(fr_ensemble *e);
 void tc_destroy(fr_ensemble *e);
 // Per-agent outputs through the tcgen05 kernels; obs rows of stride ld.
-int tc_forward(const fr_ensemble *e, const float *obs, int ld, int n, float *y, cudaStream_t s);
+// `large`: the call stands for the large-batch kernel where there is one, which
+// keeps a NaN of a hidden layer; the single-agent kernel makes it 0 (max(x, 0)).
+int tc_forward(const fr_ensemble *e, const float *obs, int ld, int n, float *y, cudaStream_t s, bool large = false);
 // FP8 activation scales sx[j][l] (host [M][L]) of an FP8 ensemble (fr_tc.cu)
 int tc_set_act_scales(fr_ensemble *e, const float *scales);
 int tc_get_act_scales(const fr_ensemble *e, float *scales);
@@ -373,16 +375,15 @@ int tc_forward_tiled(const fr_ensemble *e, const float *obs, int ld, int n, floa
 // same results as tc_forward and the fused crypto rollout.
 bool nw_ok(const fr_ensemble *e);
 int nw_prepare(const fr_ensemble *e);
-int nw_forward(const fr_ensemble *e, const float *obs, int ld, int n, float *y, cudaStream_t s);
+int nw_forward(const fr_ensemble *e, const float *obs, int ld, int n, float *y, bool nan0, cudaStream_t s);
 // two hidden layers up to 256 wide, weights resident in CTA pairs (fr_wide.cu)
 bool wd_ok(const fr_ensemble *e);
 int wd_prepare(const fr_ensemble *e);
-int wd_forward(const fr_ensemble *e, const float *obs, int ld, int n, float *y, cudaStream_t s);
+int wd_forward(const fr_ensemble *e, const float *obs, int ld, int n, float *y, bool nan0, cudaStream_t s);
 // the weighted mean of the agents' outputs in the same launch, for batches wd_act_ok takes
 bool wd_act_ok(const fr_ensemble *e, int n);
 int wd_act(const fr_ensemble *e, const float *obs, int n, float *act, cudaStream_t s);
-// Fewer 128-row tiles than SMs.  Hidden NaNs become 0 (max(x, 0)) in such
-// batches and stay NaN in larger ones.
+// Fewer 128-row tiles than SMs: batches the large-batch kernel does not take.
 inline int tc_small_batch(const fr_ensemble *e, int n) { return (int)ceil_div(n, 128) < e->ctx->sm_count; }
 // the crypto rollout; its scratch holds the value log and the pieces' step counts
 uint64_t nw_rollout_scratch(const fr_env *env, int T);

@@ -536,7 +536,7 @@ int nw_prepare(const fr_ensemble *e)
     return FR_OK;
 }
 
-int nw_forward(const fr_ensemble *e, const float *obs, int ld, int n, float *y, cudaStream_t s)
+int nw_forward(const fr_ensemble *e, const float *obs, int ld, int n, float *y, bool nan0, cudaStream_t s)
 {
     NwArgs a;
     memset(&a, 0, sizeof(a));
@@ -548,7 +548,7 @@ int nw_forward(const fr_ensemble *e, const float *obs, int ld, int n, float *y, 
     a.obs = obs;
     a.ld = ld;
     a.rows = n;
-    a.nan0 = tc_small_batch(e, n);
+    a.nan0 = nan0 ? 1 : 0;
     a.tiles = (int)ceil_div(n, a.sh.n);
     a.y = y;
     FR_CUDA(set_max_smem_once((const void *)k_narrow<false>, e->ctx->device));

@@ -595,14 +595,15 @@ int tc_get_act_scales(const fr_ensemble *e, float *scales)
     return FR_OK;
 }
 
-int tc_forward(const fr_ensemble *e, const float *obs, int ld, int n, float *y, cudaStream_t s)
+int tc_forward(const fr_ensemble *e, const float *obs, int ld, int n, float *y, cudaStream_t s, bool large)
 {
     const TcImage *t = e->tc;
     FR_CHECK(t, FR_EINVAL, "tensor-core image missing");
     FR_CHECK(t->plan.esz != 1 || t->scaled, FR_ENOTREADY,
              "FP8 ensemble needs activation scales (ensemble_set_act_scales or ensemble_calibrate_sync)");
-    if (nw_ok(e)) return nw_forward(e, obs, ld, n, y, s);
-    if (wd_ok(e)) return wd_forward(e, obs, ld, n, y, s);
+    const bool nan0 = !large || tc_small_batch(e, n);
+    if (nw_ok(e)) return nw_forward(e, obs, ld, n, y, nan0, s);
+    if (wd_ok(e)) return wd_forward(e, obs, ld, n, y, nan0, s);
     dim3 grid(ceil_div(n, 128), e->M);
     k_tc_forward<<<grid, TC_THREADS, tc_smem_bytes(t->plan), s>>>(t->plan, t->img, t->bias, t->dq, t->inv_sx,
                                                                   obs, ld, n, y, t->err);

@@ -618,7 +618,7 @@ int wd_clusters(int size, uint32_t smem, int device, int sms)
 int wd_pair(const TcPlan &p) { return p.layer[0].N > WD_UNITS || p.layer[1].N > WD_UNITS ? 2 : 1; }
 
 // y: every agent's outputs, or (act) their weighted mean.
-int wd_launch(const fr_ensemble *e, const float *obs, int ld, int n, float *y, bool act, cudaStream_t s)
+int wd_launch(const fr_ensemble *e, const float *obs, int ld, int n, float *y, bool act, bool nan0, cudaStream_t s)
 {
     const TcPlan &p = e->tc->plan;
     WdArgs a;
@@ -633,7 +633,7 @@ int wd_launch(const fr_ensemble *e, const float *obs, int ld, int n, float *y, b
     a.y = y;
     a.act = act ? 1 : 0;
     a.w = e->weights;
-    a.nan0 = tc_small_batch(e, n);
+    a.nan0 = nan0 ? 1 : 0;
     a.bulk = ld == p.layer[0].fin && ((uintptr_t)obs & 15u) == 0;
     a.pair = wd_pair(p);
     const int size = a.pair * (act ? p.M : 1), most = wd_most(p, act, e->tc->optin);
@@ -698,9 +698,9 @@ int wd_prepare(const fr_ensemble *e)
     return FR_OK;
 }
 
-int wd_forward(const fr_ensemble *e, const float *obs, int ld, int n, float *y, cudaStream_t s)
+int wd_forward(const fr_ensemble *e, const float *obs, int ld, int n, float *y, bool nan0, cudaStream_t s)
 {
-    return wd_launch(e, obs, ld, n, y, false, s);
+    return wd_launch(e, obs, ld, n, y, false, nan0, s);
 }
 
 // Combining in the same launch: a cluster holds every agent (at most eight
@@ -714,7 +714,7 @@ bool wd_act_ok(const fr_ensemble *e, int n)
 
 int wd_act(const fr_ensemble *e, const float *obs, int n, float *act, cudaStream_t s)
 {
-    return wd_launch(e, obs, e->dims[0], n, act, true, s);
+    return wd_launch(e, obs, e->dims[0], n, act, true, tc_small_batch(e, n), s);
 }
 
 }  // namespace fr

@@ -63,3 +63,26 @@ def test_captured_act_follows_new_weights(ctx, dev, n, prec):
         assert torch.equal(a, b)
         seen.append(a.clone())
     assert not torch.equal(seen[0], seen[1]) and not torch.equal(seen[1], seen[2])
+
+
+@pytest.mark.parametrize("dims", [(61, 64, 200, 30), (10, 64, 64, 3)])
+@pytest.mark.parametrize("prec", [fr.PREC_BF16, fr.PREC_FP16])
+def test_nan_rows_in_large_batches(ctx, dev, dims, prec):
+    # a NaN observation: ensemble_act_noalloc stands for the single-agent kernel
+    # (max(x, 0) makes a hidden NaN 0) whatever the batch, ensemble_act and
+    # _forward for the large-batch one (it stays) from one tile of 128 rows per SM
+    M, n = 2, 128 * ctx.sm_count
+    ens = fr.ensemble_create(ctx, dims, synth.actor_params(dims, M, seed=3), precision=prec)
+    x = torch.from_numpy(np.random.default_rng(4).standard_normal((n, dims[0])).astype(np.float32)).to(dev)
+    x[5, 1] = float("nan")
+    a, few = torch.empty(n, dims[-1], device=dev), torch.empty(100, dims[-1], device=dev)
+    big, y = torch.empty_like(a), torch.empty(M, n, dims[-1], device=dev)
+    fr.ensemble_act_noalloc(ens, x, a)
+    fr.ensemble_act_noalloc(ens, x[:100].contiguous(), few)
+    fr.ensemble_act(ens, x, big)
+    fr.ensemble_forward(ens, x, y)
+    torch.cuda.synchronize()
+    assert torch.isfinite(a).all() and torch.equal(a[:100], few)
+    keep = torch.arange(n, device=dev) != 5
+    assert torch.equal(a[keep], big[keep])
+    assert torch.isnan(big[5]).all() and torch.isnan(y[:, 5]).all()
