@@ -583,6 +583,14 @@ int wd_most(const TcPlan &p, bool act, int optin)
     return a.n;
 }
 
+// Shared memory of a launch whose operands take `layout` bytes.  The CTAs of a
+// cluster wait for each other with the SM's whole tensor memory in hand, so
+// nothing else that does may share their SMs (two clusters, each holding one
+// SM's tensor memory and waiting for the other's, would wait for ever; beside
+// the 64-row kernel's registers a CTA of the first fused crypto kernel fits):
+// they take the whole shared memory too.
+uint32_t wd_smem(uint32_t layout, int size, int optin) { return size > 1 ? (uint32_t)optin : layout + 1024u; }
+
 // Clusters of `size` CTAs the device holds at once (each CTA has an SM to
 // itself), queried once per device, size and shared memory; 0 when it holds
 // none or the query fails.
@@ -639,9 +647,9 @@ int wd_launch(const fr_ensemble *e, const float *obs, int ld, int n, float *y, b
     const int size = a.pair * (act ? p.M : 1), most = wd_most(p, act, e->tc->optin);
     a.n = most;
     FR_CUDA(set_max_smem_once((const void *)k_wide<WD_ROWS>, e->ctx->device));
-    const int clusters = wd_clusters(size, wd_layout(p, &a) + 1024u, e->ctx->device, e->ctx->sm_count);
-    FR_CHECK(clusters > 0, FR_ECUDA, "no room for clusters of %d CTAs with %u bytes of shared memory each", size,
-             wd_layout(p, &a) + 1024u);
+    const uint32_t smem = wd_smem(wd_layout(p, &a), size, e->tc->optin);
+    const int clusters = wd_clusters(size, smem, e->ctx->device, e->ctx->sm_count);
+    FR_CHECK(clusters > 0, FR_ECUDA, "no room for clusters of %d CTAs with %u bytes of shared memory each", size, smem);
     // tiles: as few rows each as spread the batch over every cluster in the
     // waves it needs anyway
     const int64_t lanes = std::max(1, act ? clusters : clusters / p.M);       // tiles in flight
@@ -652,7 +660,7 @@ int wd_launch(const fr_ensemble *e, const float *obs, int ld, int n, float *y, b
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(size * (act ? 1 : p.M) * (int)std::min<int64_t>(lanes, a.tiles)), 1, 1);
     cfg.blockDim = dim3(WD_THREADS, 1, 1);
-    cfg.dynamicSmemBytes = wd_layout(p, &a) + 1024u;
+    cfg.dynamicSmemBytes = wd_smem(wd_layout(p, &a), size, e->tc->optin);
     cfg.stream = s;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -689,11 +697,12 @@ int wd_prepare(const fr_ensemble *e)
     const TcPlan &p = e->tc->plan;
     for (auto k : wd_kernels) FR_CUDA(set_max_smem_once((const void *)k, e->ctx->device));
     a.n = wd_most(p, false, e->tc->optin);
-    wd_clusters(wd_pair(p), wd_layout(p, &a) + 1024u, e->ctx->device, e->ctx->sm_count);
+    wd_clusters(wd_pair(p), wd_smem(wd_layout(p, &a), wd_pair(p), e->tc->optin), e->ctx->device, e->ctx->sm_count);
     if (wd_act_ok(e, 1)) {
         a.act = 1;
         a.n = wd_most(p, true, e->tc->optin);
-        wd_clusters(wd_pair(p) * p.M, wd_layout(p, &a) + 1024u, e->ctx->device, e->ctx->sm_count);
+        const int size = wd_pair(p) * p.M;
+        wd_clusters(size, wd_smem(wd_layout(p, &a), size, e->tc->optin), e->ctx->device, e->ctx->sm_count);
     }
     return FR_OK;
 }

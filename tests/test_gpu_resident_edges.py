@@ -86,3 +86,33 @@ def test_nan_rows_in_large_batches(ctx, dev, dims, prec):
     keep = torch.arange(n, device=dev) != 5
     assert torch.equal(a[keep], big[keep])
     assert torch.isnan(big[5]).all() and torch.isnan(y[:, 5]).all()
+
+
+def test_forward_beside_a_fused_rollout(ctx, dev):
+    # two kernels whose CTAs work in clusters and hold tensor memory, on two
+    # streams at once: the results are those of each alone
+    dims, M, n, N, T = (10, 144, 96, 3), 5, 5000, 700, 40
+    P = synth.actor_params(dims, M, seed=8, out_scale=4.0)
+    ens = fr.ensemble_create(ctx, dims, P, precision=fr.PREC_BF16, out_act=0)
+    vote = fr.ensemble_create(ctx, dims, P, precision=fr.PREC_BF16, combine=fr.COMBINE_VOTE, out_act=0)
+    mk = fr.fr_market_create(ctx, synth.crypto_market(9_000, seed=8))
+    env = fr.env_create(ctx, mk, start=np.arange(N) % 4000 + 3600, window=T + 1, pmax=3)
+    x = torch.from_numpy(np.random.default_rng(8).standard_normal((n, dims[0])).astype(np.float32)).to(dev)
+    y = [torch.empty(M, n, dims[-1], device=dev) for _ in range(2)]
+    m = [torch.empty(N, 3, dtype=torch.float64, device=dev) for _ in range(2)]
+    s = [torch.cuda.Stream() for _ in range(2)]
+    fr.ensemble_forward(ens, x, y[0])
+    torch.cuda.synchronize()
+    fr.rollout(env, vote, T, metrics=m[0])
+    torch.cuda.synchronize()
+    for _ in range(10):
+        y[1].fill_(-7.0)
+        m[1].fill_(-7.0)
+        torch.cuda.synchronize()
+        fr.env_reset(env, stream=s[0])
+        fr.rollout(env, vote, T, metrics=m[1], stream=s[0])
+        for _ in range(20):
+            fr.ensemble_forward(ens, x, y[1], stream=s[1])
+        torch.cuda.synchronize()
+        assert torch.equal(y[0], y[1]) and torch.equal(m[0], m[1])
+    assert fr.ensemble_device_errors(ens) == 0 and fr.ensemble_device_errors(vote) == 0
