@@ -1052,7 +1052,14 @@ int tc_rollout(fr_env *env, const fr_ensemble *e, int T, const fr_traj *traj, do
     a.err = e->tc->err;
     a.ex = explore_of(env, env->explore_step);
 
-    const uint32_t smem = fused_smem(v.task, p, ring_bytes);
+    // At least the share of the SM's shared memory that its columns are of the
+    // 512 of tensor memory: a cluster's CTAs wait for each other, so none may
+    // sit on an SM where it waits for tensor memory that another cluster holds
+    // (10-144-96-3: 73 KB, three CTAs of 256 columns would fit).
+    int cap = 0;
+    FR_CUDA(cudaDeviceGetAttribute(&cap, cudaDevAttrMaxSharedMemoryPerMultiprocessor, env->ctx->device));
+    const uint32_t smem =
+        std::max(fused_smem(v.task, p, ring_bytes), (uint32_t)cap / 512u * (uint32_t)p.tmem_cols - 1024u);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)p.M, ceil_div(v.N, 128), 1);
     cfg.blockDim = dim3(FU_THREADS, 1, 1);

@@ -116,3 +116,22 @@ def test_forward_beside_a_fused_rollout(ctx, dev):
         torch.cuda.synchronize()
         assert torch.equal(y[0], y[1]) and torch.equal(m[0], m[1])
     assert fr.ensemble_device_errors(ens) == 0 and fr.ensemble_device_errors(vote) == 0
+
+
+def test_fused_crypto_rollout_of_many_clusters(ctx, dev):
+    # 256 columns of tensor memory per CTA and more clusters than the GPU holds
+    # at two CTAs per SM: the rollout equals the unfused one
+    dims, M, N, T = (10, 144, 96, 3), 5, 12_000, 12
+    ens = fr.ensemble_create(ctx, dims, synth.actor_params(dims, M, seed=8, out_scale=4.0), precision=fr.PREC_BF16,
+                             combine=fr.COMBINE_VOTE, out_act=0)
+    mk = fr.fr_market_create(ctx, synth.crypto_market(9_000, seed=8))
+    out = []
+    for path in (fr.PATH_AUTO, fr.PATH_UNFUSED):
+        env = fr.env_create(ctx, mk, start=np.arange(N) % 4000 + 3600, window=T + 1, pmax=3)
+        fr.env_set_rollout_path(env, path)
+        act, m = torch.empty(T, N, dtype=torch.uint8, device=dev), torch.empty(N, 3, dtype=torch.float64, device=dev)
+        fr.rollout(env, ens, T, traj={"act": act}, metrics=m)
+        torch.cuda.synchronize()
+        out.append((act, m))
+    assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
+    assert fr.ensemble_device_errors(ens) == 0
