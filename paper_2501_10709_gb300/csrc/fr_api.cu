@@ -50,6 +50,12 @@ int ctx_reserve(fr_ctx *ctx, uint64_t bytes)
     return FR_OK;
 }
 
+bool ctx_has_room(const fr_ctx *ctx, uint64_t freed, uint64_t bytes)
+{
+    std::lock_guard<std::mutex> lk(g_budget_mu);
+    return !ctx->budget || ctx->used - freed + bytes <= ctx->budget;
+}
+
 void ctx_release(fr_ctx *ctx, uint64_t bytes)
 {
     std::lock_guard<std::mutex> lk(g_budget_mu);

@@ -204,6 +204,8 @@ namespace fr {
 // Account `bytes` against the context budget; FR_ENOMEM when it would not fit.
 int ctx_reserve(fr_ctx *ctx, uint64_t bytes);
 void ctx_release(fr_ctx *ctx, uint64_t bytes);
+// Whether the budget has room for `bytes` in place of `freed` bytes held now.
+bool ctx_has_room(const fr_ctx *ctx, uint64_t freed, uint64_t bytes);
 // cudaMalloc with budget accounting.
 int dev_alloc(fr_ctx *ctx, void **p, uint64_t bytes);
 // true when an armed host fault injection (fr_fault_inject) fails this event
@@ -385,7 +387,8 @@ bool wd_act_ok(const fr_ensemble *e, int n);
 int wd_act(const fr_ensemble *e, const float *obs, int n, float *act, cudaStream_t s);
 // Fewer 128-row tiles than SMs: batches the large-batch kernel does not take.
 inline int tc_small_batch(const fr_ensemble *e, int n) { return (int)ceil_div(n, 128) < e->ctx->sm_count; }
-// the crypto rollout; its scratch holds the value log and the pieces' step counts
+// the crypto rollout; its scratch holds the value log and the pieces' step
+// counts (with room for the log alone it is one launch)
 uint64_t nw_rollout_scratch(const fr_env *env, int T);
 int nw_rollout(fr_env *env, const fr_ensemble *e, int T, const fr_traj *traj, void *scratch, double *metrics,
                cudaStream_t s);

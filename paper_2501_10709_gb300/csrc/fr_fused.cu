@@ -1018,7 +1018,15 @@ int tc_rollout(fr_env *env, const fr_ensemble *e, int T, const fr_traj *traj, do
     }
     // value log [T][N] in the env's scratch (grown outside any timed region)
     const bool narrow = v.task == FR_TASK_CRYPTO && nw_ok(e) && !ring;
-    const uint64_t need = narrow ? nw_rollout_scratch(env, T) : (uint64_t)T * v.N * 8;
+    uint64_t need = (uint64_t)T * v.N * 8;
+    if (narrow && env->scratch_bytes < nw_rollout_scratch(env, T)) {
+        // the pieces' step counts too, unless the budget has no room for them or
+        // a capture has to make do with what there is
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        FR_CUDA(cudaStreamIsCapturing(s, &cap));
+        if (cap == cudaStreamCaptureStatusNone && ctx_has_room(env->ctx, env->scratch_bytes, nw_rollout_scratch(env, T)))
+            need = nw_rollout_scratch(env, T);
+    }
     if (env->scratch_bytes < need) {
         FR_CUDA(cudaStreamSynchronize(s));
         dev_free(env->ctx, env->scratch, env->scratch_bytes);

@@ -599,7 +599,8 @@ int nw_rollout(fr_env *env, const fr_ensemble *e, int T, const fr_traj *traj, vo
     a.ex = explore_of(env, env->explore_step);
     const int grid = (int)ceil_div(v.N, a.sh.n);
     const bool want_traj = traj->obs || traj->act || traj->rew || traj->rew_f32 || traj->done;
-    const int K = !want_traj && !v.auto_reset && !env->split_off && grid < env->ctx->sm_count
+    const int K = !want_traj && !v.auto_reset && !env->split_off && grid < env->ctx->sm_count &&
+                          env->scratch_bytes >= nw_rollout_scratch(env, T)
                       ? std::min(SPLIT_PIECES_MAX, T / 64)
                       : 1;
     FR_CUDA(set_max_smem_once((const void *)k_narrow<true>, env->ctx->device));

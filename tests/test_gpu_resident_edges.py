@@ -135,3 +135,42 @@ def test_fused_crypto_rollout_of_many_clusters(ctx, dev):
         out.append((act, m))
     assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
     assert fr.ensemble_device_errors(ens) == 0
+
+
+def test_narrow_rollout_with_room_for_the_log_alone(dev):
+    # the step counts of a rollout in pieces are no reason to refuse one: not
+    # under a budget with room for the value log alone, nor in a capture of an
+    # env whose scratch is that log
+    N, T, dims, M = 300, 200, (10, 64, 64, 3), 3
+
+    def setup(budget):
+        ctx = fr.fr_ctx_create(0, budget)
+        mk = fr.fr_market_create(ctx, synth.crypto_market(9_000, seed=8))
+        env = fr.env_create(ctx, mk, start=np.arange(N) % 4000 + 3600, window=T + 1, pmax=3)
+        kw = dict(combine=fr.COMBINE_VOTE, out_act=0)
+        P = synth.actor_params(dims, M, seed=8, out_scale=4.0)
+        ens = fr.ensemble_create(ctx, dims, P, precision=fr.PREC_FP16, **kw)
+        x3 = fr.ensemble_create(ctx, dims, P, precision=fr.PREC_BF16X3, **kw)
+        return ctx, mk, env, ens, x3, torch.empty(N, 3, dtype=torch.float64, device=dev)
+
+    free = setup(0)
+    fr.rollout(free[2], free[3], T, metrics=free[5])
+    probe = setup(1 << 30)
+    with pytest.raises(fr.FrError, match="in use") as err:
+        fr.replay_create(probe[0], probe[2], 1 << 30)
+    used = int(str(err.value).split("exceeded: ")[1].split(" in use")[0])
+    tight = setup(used + 8 * N * T)
+    fr.rollout(tight[2], tight[3], T, metrics=tight[5])
+    torch.cuda.synchronize()
+    assert torch.equal(free[5], tight[5])
+    # captured: the first fused kernel's rollout has made the scratch one value log
+    ctx, mk, env, ens, x3, m = setup(0)
+    fr.rollout(env, x3, T, metrics=m)
+    torch.cuda.synchronize()
+    g, side = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    with torch.cuda.graph(g, stream=side):
+        fr.env_reset(env, stream=side)
+        fr.rollout(env, ens, T, metrics=m, stream=side)
+    g.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(free[5], m)
