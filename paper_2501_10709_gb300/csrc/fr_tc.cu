@@ -539,9 +539,10 @@ int tc_create(fr_ensemble *e)
         err = cudaFuncSetAttribute(k_tc_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
     e->tc = t;
     if (err != cudaSuccess) return cuda_fail(err, "tc_create upload");
-    if (nw_ok(e)) return nw_prepare(e);
-    if (wd_ok(e)) return wd_prepare(e);
-    return FR_OK;
+    // (a narrow MEAN ensemble forwards in the one and acts in the other)
+    int ready = nw_ok(e) ? nw_prepare(e) : FR_OK;
+    if (!ready && wd_ok(e)) ready = wd_prepare(e);
+    return ready;
 }
 
 void tc_destroy(fr_ensemble *e)

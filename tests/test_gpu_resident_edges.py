@@ -174,3 +174,23 @@ def test_narrow_rollout_with_room_for_the_log_alone(dev):
     g.replay()
     torch.cuda.synchronize()
     assert torch.equal(free[5], m)
+
+
+def test_first_call_of_a_narrow_mean_ensemble_inside_a_capture(ctx, dev):
+    # its forward and its act run different kernels, both prepared with it
+    dims, M, n = (10, 128, 128, 3), 2, 70
+    ens = fr.ensemble_create(ctx, dims, synth.actor_params(dims, M, seed=9), precision=fr.PREC_BF16)
+    x, y, a = torch.zeros(n, dims[0], device=dev), torch.empty(M, n, 3, device=dev), torch.empty(n, 3, device=dev)
+    torch.cuda.synchronize()
+    g, side = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    with torch.cuda.graph(g, stream=side):
+        fr.ensemble_forward(ens, x, y, stream=side)
+        fr.ensemble_act(ens, x, a, stream=side)
+    for seed in range(2):
+        x.copy_(torch.from_numpy(np.random.default_rng(seed).standard_normal((n, dims[0])).astype(np.float32)))
+        g.replay()
+        y2, a2 = torch.empty_like(y), torch.empty_like(a)
+        fr.ensemble_forward(ens, x, y2)
+        fr.ensemble_act(ens, x, a2)
+        torch.cuda.synchronize()
+        assert torch.equal(y, y2) and torch.equal(a, a2)
