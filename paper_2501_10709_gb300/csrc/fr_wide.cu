@@ -239,8 +239,13 @@ __device__ __forceinline__ void wd_combine(const WdArgs &a, WdBars *bars, uint8_
 
 // n: rows per tile, at compile time: descriptors that advance by constants cost
 // the issuing warp less than its MMAs (77,824 rows: 139 us, 153 us with n a
-// parameter).
-template <int n>
+// parameter).  QUADS: input widths that are a multiple of 4, whose staged rows
+// are read 16 bytes at a time: one float at a time, the four rows of a width of
+// 200 or 304 fall on the same banks (forward on 77,824 rows: 3 x 304-256-256-30
+// 237 -> 162 us, 3 x 64-256-256-30 105 -> 102 us; inputs up to 32 wide are as
+// fast without, 3 x 16-256-256-30 95 us and 100 us with).  At compile time: both
+// forms in one kernel cost the odd widths 10 us of 127.
+template <int n, bool QUADS>
 __global__ void __launch_bounds__(WD_THREADS, 1) k_wide(const __grid_constant__ WdArgs a)
 {
     using namespace ptx;
@@ -446,8 +451,15 @@ __global__ void __launch_bounds__(WD_THREADS, 1) k_wide(const __grid_constant__ 
                 const uint32_t at = xs + (uint32_t)b * a.x_bytes + (uint32_t)(r / 8) * 128u + (uint32_t)(r % 8) * 16u;
                 for (int ch = lane >> 2; ch < chunks; ch += 8) {
                     float x[8];
+                    if constexpr (QUADS) {
 #pragma unroll
-                    for (int u = 0; u < 8; ++u) x[u] = ch * 8 + u < fin ? src[ch * 8 + u] : 0.0f;
+                        for (int u = 0; u < 8; u += 4)
+                            *(float4 *)(x + u) = ch * 8 + u < fin ? *(const float4 *)(src + ch * 8 + u)
+                                                                  : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                    } else {
+#pragma unroll
+                        for (int u = 0; u < 8; ++u) x[u] = ch * 8 + u < fin ? src[ch * 8 + u] : 0.0f;
+                    }
                     uint32_t v[4];
                     pack8_16(x, v, f16);
                     st_shared_v4(at + (uint32_t)ch * xcol, v[0], v[1], v[2], v[3]);
@@ -545,7 +557,14 @@ __global__ void __launch_bounds__(WD_THREADS, 1) k_wide(const __grid_constant__ 
     if (size > 1) cluster_sync_all();                      // no peer touches this CTA's memory after it exits
 }
 
-void (*const wd_kernels[4])(const WdArgs) = {k_wide<16>, k_wide<32>, k_wide<48>, k_wide<64>};   // by rows / 16
+// by 4-float rows, rows / 16
+void (*const wd_kernels[2][4])(const WdArgs) = {
+    {k_wide<16, false>, k_wide<32, false>, k_wide<48, false>, k_wide<64, false>},
+    {k_wide<16, true>, k_wide<32, true>, k_wide<48, true>, k_wide<64, true>}};
+auto wd_kernel(const TcPlan &p, int rows)
+{
+    return wd_kernels[p.layer[0].fin % 4 == 0 && p.layer[0].fin > 32][rows / 16 - 1];
+}
 
 // Shared memory of a launch (bytes, without the alignment slack).  The hidden
 // operand of the output layer comes first: its M = 64 rows read past a shorter
@@ -614,7 +633,7 @@ int wd_clusters(int size, uint32_t smem, int device, int sms)
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, k_wide<WD_ROWS>, &cfg) != cudaSuccess || n < 1) {
+    if (cudaOccupancyMaxActiveClusters(&n, k_wide<WD_ROWS, false>, &cfg) != cudaSuccess || n < 1) {
         cudaGetLastError();
         return 0;
     }
@@ -646,7 +665,7 @@ int wd_launch(const fr_ensemble *e, const float *obs, int ld, int n, float *y, b
     a.pair = wd_pair(p);
     const int size = a.pair * (act ? p.M : 1), most = wd_most(p, act, e->tc->optin);
     a.n = most;
-    FR_CUDA(set_max_smem_once((const void *)k_wide<WD_ROWS>, e->ctx->device));
+    FR_CUDA(set_max_smem_once((const void *)k_wide<WD_ROWS, false>, e->ctx->device));
     const uint32_t smem = wd_smem(wd_layout(p, &a), size, e->tc->optin);
     const int clusters = wd_clusters(size, smem, e->ctx->device, e->ctx->sm_count);
     FR_CHECK(clusters > 0, FR_ECUDA, "no room for clusters of %d CTAs with %u bytes of shared memory each", size, smem);
@@ -672,8 +691,8 @@ int wd_launch(const fr_ensemble *e, const float *obs, int ld, int n, float *y, b
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    FR_CUDA(set_max_smem_once((const void *)wd_kernels[a.n / 16 - 1], e->ctx->device));
-    FR_CUDA(cudaLaunchKernelEx(&cfg, wd_kernels[a.n / 16 - 1], a));
+    FR_CUDA(set_max_smem_once((const void *)wd_kernel(p, a.n), e->ctx->device));
+    FR_CUDA(cudaLaunchKernelEx(&cfg, wd_kernel(p, a.n), a));
     return FR_OK;
 }
 
@@ -695,7 +714,8 @@ int wd_prepare(const fr_ensemble *e)
     WdArgs a;
     memset(&a, 0, sizeof(a));
     const TcPlan &p = e->tc->plan;
-    for (auto k : wd_kernels) FR_CUDA(set_max_smem_once((const void *)k, e->ctx->device));
+    FR_CUDA(set_max_smem_once((const void *)k_wide<WD_ROWS, false>, e->ctx->device));   // the occupancy query's
+    for (int r = 16; r <= WD_ROWS; r += 16) FR_CUDA(set_max_smem_once((const void *)wd_kernel(p, r), e->ctx->device));
     a.n = wd_most(p, false, e->tc->optin);
     wd_clusters(wd_pair(p), wd_smem(wd_layout(p, &a), wd_pair(p), e->tc->optin), e->ctx->device, e->ctx->sm_count);
     if (wd_act_ok(e, 1)) {

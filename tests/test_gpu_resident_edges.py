@@ -194,3 +194,27 @@ def test_first_call_of_a_narrow_mean_ensemble_inside_a_capture(ctx, dev):
         fr.ensemble_act(ens, x, a2)
         torch.cuda.synchronize()
         assert torch.equal(y, y2) and torch.equal(a, a2)
+
+
+@pytest.mark.parametrize("dims,M", [((32, 160, 160, 30), 2), ((36, 200, 40, 17), 3), ((64, 64, 64, 30), 1),
+                                    ((100, 256, 129, 30), 2), ((200, 64, 64, 30), 3), ((300, 256, 256, 30), 2)])
+@pytest.mark.parametrize("prec", ["fp16", "bf16"])
+def test_input_widths_of_whole_quads(ctx, dev, dims, M, prec):
+    # rows read 16 bytes at a time: the last quad of the width, packed rows and
+    # rows at any address
+    f16 = prec == "fp16"
+    P = synth.actor_params(dims, M, seed=sum(dims))
+    ens = fr.ensemble_create(ctx, dims, P, precision=fr.PREC_FP16 if f16 else fr.PREC_BF16)
+    for n in (1, 5, 65, 2500):
+        x = np.random.default_rng(n).standard_normal((n, dims[0])).astype(np.float32)
+        xd = torch.from_numpy(x).to(dev)
+        z = torch.empty(n * dims[0] + 1, device=dev)[1:].view(n, dims[0])
+        z.copy_(xd)
+        y, y2 = torch.empty(M, n, dims[-1], device=dev), torch.empty(M, n, dims[-1], device=dev)
+        fr.ensemble_forward(ens, xd, y)
+        fr.ensemble_forward(ens, z, y2)
+        torch.cuda.synchronize()
+        assert torch.equal(y, y2)
+        for j in range(M):
+            want, err = _forward16(dims, P[j], x.astype(np.float64), f16, 1)
+            assert (np.abs(y[j].cpu().numpy() - want) <= err).all()
