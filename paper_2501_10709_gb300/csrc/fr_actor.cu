@@ -842,7 +842,7 @@ int ta_stages(const TcPlan &p, int optin, uint32_t *stage_bytes)
 uint64_t tc_tiled_scratch_bytes(const fr_ensemble *e, int n)
 {
     if (!e->tc || e->tc->plan.split != 1) return 0;                          // BF16 or FP8, not split
-    if (nw_ok(e) || wd_ok(e)) return 0;                                      // resident-weight kernels take every size
+    if (nw_ok(e) || (wd_ok(e) && wd_batch(e, n))) return 0;                  // resident-weight kernels
     // FP8: one observation tile serves every agent, so they must share the
     // layer-0 activation scale (calibration always gives them the same)
     if (e->tc->plan.esz == 1 && !(e->tc->scaled && e->tc->shared_l0)) return 0;

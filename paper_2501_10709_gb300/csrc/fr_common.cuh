@@ -380,6 +380,7 @@ int nw_prepare(const fr_ensemble *e);
 int nw_forward(const fr_ensemble *e, const float *obs, int ld, int n, float *y, bool nan0, cudaStream_t s);
 // two hidden layers up to 256 wide, weights resident in CTA pairs (fr_wide.cu)
 bool wd_ok(const fr_ensemble *e);
+bool wd_batch(const fr_ensemble *e, int n);    // and as fast there as the large-batch kernel on n rows
 int wd_prepare(const fr_ensemble *e);
 int wd_forward(const fr_ensemble *e, const float *obs, int ld, int n, float *y, bool nan0, cudaStream_t s);
 // the weighted mean of the agents' outputs in the same launch, for batches wd_act_ok takes

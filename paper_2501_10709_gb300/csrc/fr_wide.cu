@@ -707,6 +707,34 @@ bool wd_ok(const fr_ensemble *e)
            p.layer[1].N <= 256 && p.layer[1].K <= 256 && p.layer[2].K <= 256 && p.layer[2].N <= 32;
 }
 
+// Whether a forward of n rows of a network wd_ok takes runs here, where the
+// tiled large-batch kernel could (from one 128-row tile per SM): the faster by
+// this estimate of both, in us per 77,824 rows (four waves of the tiled kernel's
+// tiles).  A row here costs much the same whatever its hidden layers' widths
+// (26 us per agent over CTA pairs, 15.5 in single CTAs, 4 for more than 16
+// outputs, and the loading), while the tiled kernel, which converts the rows
+// once for every agent, pays for the columns that there are and for whole waves.
+// Fitted to 560 shapes at 19,455 .. 262,144 rows; what it picks is at most 5%
+// behind the better one (3 x 10-144-96-3 on 262,144 rows: 212 us tiled, 258
+// here; 8 x 304-16-256-30 on 77,824: 267 and 410; 3 x 301-256-256-30: 164 and
+// 127).
+bool wd_batch(const fr_ensemble *e, int n)
+{
+    if (tc_small_batch(e, n)) return true;
+    const TcPlan &p = e->tc->plan;
+    const int fin = p.layer[0].fin, sms = e->ctx->sm_count;
+    const double K = p.layer[0].K, tiles = ceil_div(n, 128), outs = p.layer[2].N > 16 ? 1.0 : 0.0;
+    const double rows = (double)WD_ROWS / wd_most(p, false, e->tc->optin);
+    const double agent = 4.0 * outs + (wd_pair(p) == 2 ? 26.0 + 0.03 * K : 15.5 + 0.012 * K);
+    double tiled = 13.0 + 5.0 * outs;
+    for (int l = 0; l < 2; ++l)
+        tiled += (p.layer[l].N > 128 ? 4.0 : 0.0) + p.layer[l].K * p.layer[l].N / 10200.0;
+    // the tiling pass reads rows that share banks at multiples of 16 and 32
+    const double pass = 2.0 + K * (fin % 32 == 0 ? 0.26 : fin % 16 == 0 ? 0.18 : 0.09);
+    return 4.0 + (0.02 * K + p.M * agent * rows) * tiles / (4.0 * sms) <=
+           13.0 + (pass + p.M * tiled) * ceil_div((long long)tiles, sms) / 4.0;
+}
+
 // The host queries and kernel attributes of every launch shape, so that a
 // first call may be inside a stream capture.
 int wd_prepare(const fr_ensemble *e)

@@ -218,3 +218,30 @@ def test_input_widths_of_whole_quads(ctx, dev, dims, M, prec):
         for j in range(M):
             want, err = _forward16(dims, P[j], x.astype(np.float64), f16, 1)
             assert (np.abs(y[j].cpu().numpy() - want) <= err).all()
+
+
+@pytest.mark.parametrize("dims,M", [((10, 144, 96, 3), 5), ((61, 64, 64, 30), 8), ((128, 16, 256, 30), 4),
+                                    ((304, 129, 256, 30), 8), ((301, 128, 256, 17), 6)])
+@pytest.mark.parametrize("prec", [fr.PREC_BF16, fr.PREC_FP16])
+def test_large_batches_on_either_kernel(ctx, dev, dims, M, prec):
+    # around the lines where large batches change between the resident and the
+    # tiled kernel (a wave of tiles more, the last wave nearly empty or full):
+    # every row as in a small batch, acts as forward then mean
+    ens = fr.ensemble_create(ctx, dims, synth.actor_params(dims, M, seed=sum(dims)), precision=prec)
+    wave = 128 * ctx.sm_count
+    x = torch.from_numpy(np.random.default_rng(6).standard_normal((2 * wave + 3, dims[0])).astype(np.float32)).to(dev)
+    few = torch.empty(M, 2000, dims[-1], device=dev)
+    w = torch.full((), np.float32(1.0 / M).item(), device=dev)
+    for n in (wave - 128, wave - 127, wave, wave + 1, 2 * wave - 1, 2 * wave + 3):
+        y, act = torch.empty(M, n, dims[-1], device=dev), torch.empty(n, dims[-1], device=dev)
+        fr.ensemble_forward(ens, x[:n].contiguous(), y)
+        fr.ensemble_act(ens, x[:n].contiguous(), act)
+        for r in (0, n - 2000):
+            fr.ensemble_forward(ens, x[r:r + 2000].contiguous(), few)
+            torch.cuda.synchronize()
+            assert torch.equal(y[:, r:r + 2000], few)
+        want = y[0].clone()
+        for j in range(1, M):
+            want = want + w * (y[j] - y[0])
+        assert torch.equal(act, want)
+    assert fr.ensemble_device_errors(ens) == 0
