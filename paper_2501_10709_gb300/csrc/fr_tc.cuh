@@ -63,6 +63,7 @@ struct TcImage {
     unsigned *err;        // device error flags
     uint64_t bytes;
     int optin = 0;        // most shared memory of a block on the device
+    int act_rows = 0;     // largest batch whose agents one launch combines (fr_wide.cu)
     // FP8 only: dequantisation factors sx[l] * sw[n] [M][MAX_LAYERS][256] and
     // the inverse activation scales 1 / sx[l] [M][MAX_LAYERS] (device); the
     // scales themselves (host) and whether activation scales were set

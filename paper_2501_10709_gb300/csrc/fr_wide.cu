@@ -63,7 +63,7 @@ constexpr int WD_MMA_WARP = 12 + WD_LOADERS;
 constexpr int WD_THREADS = 32 * (WD_MMA_WARP + 1);
 constexpr int WD_GROUP = 4;                       // rows a loader warp stages at a time: 16 ld bytes apart, so
                                                   // every group of an aligned batch starts on a 16-byte boundary
-constexpr int WD_ACT_MAX = 4096;                  // most rows combined in the same launch
+constexpr int WD_ACT_MAX = 4096, WD_ACT_WAVES = 2;   // most rows, and waves of tiles, combined in the same launch
 constexpr int WD_ACT_ROWS = 48;                   // most rows of a tile where the agents are combined
 constexpr uint32_t WD_ACC2 = 64u, WD_OUT = 128u, WD_W1 = 160u;   // tensor memory columns
 
@@ -746,11 +746,21 @@ int wd_prepare(const fr_ensemble *e)
     for (int r = 16; r <= WD_ROWS; r += 16) FR_CUDA(set_max_smem_once((const void *)wd_kernel(p, r), e->ctx->device));
     a.n = wd_most(p, false, e->tc->optin);
     wd_clusters(wd_pair(p), wd_smem(wd_layout(p, &a), wd_pair(p), e->tc->optin), e->ctx->device, e->ctx->sm_count);
-    if (wd_act_ok(e, 1)) {
+    // Combining in the same launch: a cluster holds every agent (at most eight
+    // CTAs), 48 rows a tile.  It spares small batches, which wait for the host,
+    // an allocation and a launch (8 rows of 3 x 301-256-256-30: 12.3 us a call),
+    // but the GPU holds few such clusters (23 of six, 14 of eight), so that past
+    // two waves of them a forward over every SM and a combining launch are faster
+    // on the GPU by more than they cost the host: 8 x 61-64-64-30 on 4,096 rows
+    // 54 us combined, 20 us in two launches; 3 x 301-256-256-30 on 3,072 rows 24
+    // and 17, on 2,048 rows (two waves) 17.4 and 17.1.
+    const int size = wd_pair(p) * p.M;
+    if (e->combine == FR_COMBINE_MEAN && size <= 8) {
         a.act = 1;
         a.n = wd_most(p, true, e->tc->optin);
-        const int size = wd_pair(p) * p.M;
-        wd_clusters(size, wd_smem(wd_layout(p, &a), size, e->tc->optin), e->ctx->device, e->ctx->sm_count);
+        const int clusters =
+            wd_clusters(size, wd_smem(wd_layout(p, &a), size, e->tc->optin), e->ctx->device, e->ctx->sm_count);
+        e->tc->act_rows = std::min(WD_ACT_MAX, WD_ACT_WAVES * a.n * clusters);
     }
     return FR_OK;
 }
@@ -760,14 +770,7 @@ int wd_forward(const fr_ensemble *e, const float *obs, int ld, int n, float *y, 
     return wd_launch(e, obs, ld, n, y, false, nan0, s);
 }
 
-// Combining in the same launch: a cluster holds every agent (at most eight
-// CTAs).  23 clusters of six fit the GPU with 48 rows each, 25 pairs per agent
-// with 64: past four waves of the former a forward and a combining launch are
-// as fast.
-bool wd_act_ok(const fr_ensemble *e, int n)
-{
-    return wd_ok(e) && e->combine == FR_COMBINE_MEAN && wd_pair(e->tc->plan) * e->M <= 8 && n <= WD_ACT_MAX;
-}
+bool wd_act_ok(const fr_ensemble *e, int n) { return e->tc && n <= e->tc->act_rows; }
 
 int wd_act(const fr_ensemble *e, const float *obs, int n, float *act, cudaStream_t s)
 {

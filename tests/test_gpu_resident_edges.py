@@ -245,3 +245,24 @@ def test_large_batches_on_either_kernel(ctx, dev, dims, M, prec):
             want = want + w * (y[j] - y[0])
         assert torch.equal(act, want)
     assert fr.ensemble_device_errors(ens) == 0
+
+
+@pytest.mark.parametrize("dims,M", [((61, 64, 64, 30), 8), ((10, 16, 16, 3), 6), ((301, 256, 256, 30), 4), ((61, 64, 64, 30), 1)])
+def test_act_around_its_waves(ctx, dev, dims, M):
+    # batch sizes around the line between the agents combined in the forward's
+    # launch and after it: the same actions
+    w = np.random.default_rng(M).random(M).astype(np.float32)
+    ens = fr.ensemble_create(ctx, dims, synth.actor_params(dims, M, seed=M), weights=w, precision=fr.PREC_BF16)
+    wt = torch.from_numpy(w).to(dev)
+    x = torch.from_numpy(np.random.default_rng(3).standard_normal((4100, dims[0])).astype(np.float32)).to(dev)
+    y = torch.empty(M, 4100, dims[-1], device=dev)
+    fr.ensemble_forward(ens, x, y)
+    want = y[0].clone()
+    for j in range(1, M):
+        want = want + wt[j] * (y[j] - y[0])
+    for n in (1, *range(96 * 10, 4100, 191), 4095, 4096, 4097):
+        act = torch.full((n + 1, dims[-1]), -7.0, device=dev)
+        fr.ensemble_act(ens, x[:n].contiguous(), act[:n])
+        torch.cuda.synchronize()
+        assert torch.equal(act[:n], want[:n]) and (act[n] == -7.0).all()
+    assert fr.ensemble_device_errors(ens) == 0
