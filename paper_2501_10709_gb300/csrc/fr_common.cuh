@@ -402,6 +402,9 @@ bool tc_rollout_supported(const fr_env *env, const fr_ensemble *e);
 // writes them (its count restarts with every episode, as the kernel's).
 cudaError_t launch_metrics_replay(const EnvView &v, const int64_t *vlog, int T, double *metrics,
                                   cudaStream_t s, const int32_t *t0 = nullptr);
+// whether one thread per env is the faster form (fr_metrics.cu) for the replay of
+// a log, or (traj) the metrics of stored trajectories, of T steps of N envs
+bool episodes_short(bool traj, int T, int N);
 // its form without auto-reset (fr_metrics.cu): every env's logged steps are a
 // prefix of the log, which ends with its episode
 cudaError_t launch_episode_replay(const EnvView &v, const int64_t *vlog, int T, double *metrics, cudaStream_t s,

@@ -1096,8 +1096,8 @@ int tc_rollout(fr_env *env, const fr_ensemble *e, int T, const fr_traj *traj, do
 cudaError_t launch_metrics_replay(const EnvView &v, const int64_t *vlog, int T, double *metrics,
                                   cudaStream_t s, const int32_t *t0)
 {
-    if (!v.auto_reset) return launch_episode_replay(v, vlog, T, metrics, s, t0);
-    // auto-reset: one thread per env, spread over every SM: the replay is
+    if (!v.auto_reset && !episodes_short(false, T, v.N)) return launch_episode_replay(v, vlog, T, metrics, s, t0);
+    // auto-reset, or a short log: one thread per env, spread over every SM: the replay is
     // bound by the FP64 units, and 2,048 envs in blocks of 256 would use 8 SMs
     const int per_block = std::min(256, std::max(16, (int)ceil_div(v.N, 152) + 15) / 16 * 16);
     k_metrics_replay<<<ceil_div(v.N, per_block), per_block, 0, s>>>(v, vlog, T, metrics, t0);

@@ -26,6 +26,8 @@
 // thread per env and three divisions per step in series, 77 us now; the
 // replay of 8,192 envs x 1,024 steps 1.56 ms with the mean's division on the
 // chain and the returns' beside it, 0.44 ms now (FP64 pipe 76% busy).
+#include <algorithm>
+
 #include "fr_common.cuh"
 #include "fr_env_dev.cuh"
 #include "fr_fp64.cuh"
@@ -389,6 +391,55 @@ __global__ void __launch_bounds__(EP_THREADS, 1) k_episodes(const __grid_constan
     }
 }
 
+// Trajectories that episodes_short() takes: one thread per env, step by step,
+// with plain divisions (a warp alone waits 6% less for one of them than for the
+// six operations in its place, and many warps fill the pipe either way).
+__global__ void __launch_bounds__(128) k_episodes_short(const __grid_constant__ EpArgs a)
+{
+    const int e = blockIdx.x * 128 + threadIdx.x;
+    if (e >= a.N) return;
+    double mu = 0.0, m2 = 0.0, mdd = 0.0, down2 = 0.0, up = 0.0, dn = 0.0, disc = 0.0, g = 1.0;
+    int64_t peak = a.v0, v = a.v0;
+    int n = 0;
+    for (int t = 0; t < a.T; ++t) {
+        const int64_t r = __ldg(a.in + (int64_t)t * a.N + e), v1 = v + r;
+        const double rho = __dsub_rn(__ddiv_rn((double)v1, (double)v), 1.0);
+        n += 1;
+        const double delta = __dsub_rn(rho, mu);
+        mu = __dadd_rn(mu, __ddiv_rn(delta, (double)n));
+        m2 = __dadd_rn(m2, __dmul_rn(delta, __dsub_rn(rho, mu)));
+        if (v1 > peak) peak = v1;
+        if (v1 < peak) {
+            const double dd = __dsub_rn(__ddiv_rn((double)v1, (double)peak), 1.0);
+            if (dd < mdd) mdd = dd;
+        }
+        if (rho < 0.0) {
+            down2 = __dadd_rn(down2, __dmul_rn(rho, rho));
+            dn = __dadd_rn(dn, -rho);
+        } else {
+            up = __dadd_rn(up, rho);
+        }
+        g = __dmul_rn(g, a.gamma);
+        disc = __dadd_rn(disc, __dmul_rn(g, (double)r));
+        v = v1;
+        if (a.done && __ldg(a.done + (int64_t)t * a.N + e)) break;
+    }
+    double *o = a.out + (int64_t)e * FR_TRAJ_METRICS;
+    acc_final(mu, m2, mdd, v, a.v0, n, a.ann, o);
+    const double nd = (double)n, cr = o[0], dd_max = -mdd;
+    const double annual =
+        n > 0 ? __dsub_rn(pow(__ddiv_rn((double)v, (double)a.v0), __ddiv_rn(a.ann, nd)), 1.0) : 0.0;
+    const double ddown = n > 0 ? __dsqrt_rn(__ddiv_rn(down2, nd)) : 0.0;
+    o[3] = annual;
+    o[4] = n >= 2 ? __dmul_rn(__dsqrt_rn(__ddiv_rn(m2, __dsub_rn(nd, 1.0))), __dsqrt_rn(a.ann)) : 0.0;
+    o[5] = dd_max != 0.0 ? __ddiv_rn(cr, dd_max) : 0.0;
+    o[6] = ddown != 0.0 ? __dmul_rn(__ddiv_rn(mu, ddown), __dsqrt_rn(a.ann)) : 0.0;
+    o[7] = dd_max != 0.0 ? __ddiv_rn(annual, dd_max) : 0.0;
+    o[8] = dn != 0.0 ? __ddiv_rn(up, dn) : 0.0;
+    o[9] = disc;
+    o[10] = nd;
+}
+
 // 16 envs per block while that leaves at most one block per SM (a block's
 // mean chain then has its sub-partition to itself: 260 cycles a step); 32
 // beyond, where the FP64 pipes are the limit and full warps halve the sums'
@@ -398,7 +449,9 @@ constexpr int EP_SMS = 152;
 template <bool TRAJ>
 cudaError_t launch_episodes(const EpArgs &a, cudaStream_t s)
 {
-    if (a.N <= 16 * EP_SMS)
+    if (TRAJ && episodes_short(true, a.T, a.N))
+        k_episodes_short<<<ceil_div(a.N, 128), 128, 0, s>>>(a);
+    else if (a.N <= 16 * EP_SMS)
         k_episodes<TRAJ, 16><<<ceil_div(a.N, 16), EP_THREADS, 0, s>>>(a);
     else
         k_episodes<TRAJ, 32><<<ceil_div(a.N, 32), EP_THREADS, 0, s>>>(a);
@@ -406,6 +459,22 @@ cudaError_t launch_episodes(const EpArgs &a, cudaStream_t s)
 }
 
 }  // namespace
+
+// Few steps of many envs: a block of k_episodes fills and drains its pipeline
+// for 32 envs, one block per SM, which costs a wave of them 10 us (4 the replay)
+// before its 0.27 us a step; a thread per env waits 1.65 us a step (1.2 the
+// replay) and, past a block of 128 per SM, the FP64 pipe has 1.57 us a step of
+// work for each (7.6 at 131,072 envs the replay).  The faster by these figures.
+// Trajectories of 131,072 envs x 1 step take 70 us, 280 us by k_episodes; x 64
+// steps 774 and 740; 8,192 envs x 4 steps 19 and 23, x 8 steps 26 and 26.
+bool episodes_short(bool traj, int T, int N)
+{
+    const double waves = ceil_div(ceil_div(N, N <= 16 * EP_SMS ? 16 : 32), EP_SMS);
+    if (traj)
+        return T <= 1 || std::max(12.0 + 1.65 * T, ceil_div(N, 128 * EP_SMS) * (9.4 + 1.57 * T)) <
+                             waves * (10.4 + 0.27 * T);
+    return std::max(0.4 + 1.2 * T, N / 131072.0 * (12.0 + 7.6 * T)) < waves * (4.4 + 0.27 * T);
+}
 
 cudaError_t launch_episode_replay(const EnvView &v, const int64_t *vlog, int T, double *metrics, cudaStream_t s,
                                   const int32_t *t0)
