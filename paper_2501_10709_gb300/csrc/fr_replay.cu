@@ -12,8 +12,8 @@
 // Push: the rows of a trajectory in (t, env) order; row (t, e) is a real
 // step unless the env was already done before it (done[t-1][e], or not live
 // at the start of the rollout), which frozen envs show without auto-reset.
-// Valid rows are appended in that order: a count kernel (one block per 256
-// rows), a one-block scan that also advances the device counter, and a
+// Valid rows are appended in that order: a count kernel (one block per 32 or
+// 256 rows), a one-block scan that also advances the device counter, and a
 // scatter kernel that ranks its rows again and copies them, one warp per
 // row so that every copy is coalesced.  s' of row (t, e) is obs[t+1][e], or
 // the caller's observation after the rollout for t = T - 1.
@@ -28,9 +28,6 @@
 namespace fr {
 namespace {
 
-constexpr int RP_ROWS = 256;          // rows per count / scatter block (131,072 rows of 301: 131 us with 128
-                                      // blocks of 1,024 rows, 107 us with 512 of these)
-
 __device__ __forceinline__ bool rp_valid(int64_t r, int N, const uint8_t *done, const uint8_t *live0,
                                          int auto_reset)
 {
@@ -40,10 +37,11 @@ __device__ __forceinline__ bool rp_valid(int64_t r, int N, const uint8_t *done, 
     return done[r - N] == 0;
 }
 
-__global__ void __launch_bounds__(RP_ROWS) k_rp_count(int64_t rows, int N, const uint8_t *done,
+template <int ROWS>
+__global__ void __launch_bounds__(ROWS) k_rp_count(int64_t rows, int N, const uint8_t *done,
                                                       const uint8_t *live0, int auto_reset, int64_t *counts)
 {
-    const int64_t r = (int64_t)blockIdx.x * RP_ROWS + threadIdx.x;
+    const int64_t r = (int64_t)blockIdx.x * ROWS + threadIdx.x;
     const int v = r < rows && rp_valid(r, N, done, live0, auto_reset);
     const int c = __syncthreads_count(v);
     if (threadIdx.x == 0) counts[blockIdx.x] = c;
@@ -123,28 +121,28 @@ __device__ __forceinline__ void rp_copy2(float *dst, const float *src, float *nd
     }
 }
 
-__global__ void __launch_bounds__(RP_ROWS) k_rp_scatter(RpBuf b, int64_t rows, int N, int ld, const float *obs,
+template <int ROWS, int THREADS>
+__global__ void __launch_bounds__(THREADS) k_rp_scatter(RpBuf b, int64_t rows, int N, int ld, const float *obs,
                                                         const void *act, const float *rew, const uint8_t *done,
-                                                        const float *last_obs, const uint8_t *live0,
-                                                        int auto_reset, const int64_t *offsets,
-                                                        const int64_t *state)
+                                                        const float *last_obs, const uint8_t *live0, int auto_reset,
+                                                        const int64_t *offsets, const int64_t *state)
 {
-    __shared__ int64_t slot_s[RP_ROWS];
-    __shared__ int wcount[RP_ROWS / 32];
+    __shared__ int64_t slot_s[ROWS];
+    __shared__ int wcount[ROWS / 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t r0 = (int64_t)blockIdx.x * RP_ROWS;
+    const int64_t r0 = (int64_t)blockIdx.x * ROWS;
     const int64_t r = r0 + threadIdx.x;
-    const bool v = r < rows && rp_valid(r, N, done, live0, auto_reset);
+    const bool v = (int)threadIdx.x < ROWS && r < rows && rp_valid(r, N, done, live0, auto_reset);
     const unsigned m = __ballot_sync(0xffffffffu, v);
-    if (lane == 0) wcount[warp] = __popc(m);
+    if (warp < ROWS / 32 && lane == 0) wcount[warp] = __popc(m);
     __syncthreads();
     int before = 0;
-    for (int w = 0; w < warp; ++w) before += wcount[w];
+    for (int w = 0; w < min(warp, ROWS / 32); ++w) before += wcount[w];
     const int rank = before + __popc(m & ((1u << lane) - 1u));
-    slot_s[threadIdx.x] = v ? (state[1] + offsets[blockIdx.x] + rank) % b.C : -1;
+    if ((int)threadIdx.x < ROWS) slot_s[threadIdx.x] = v ? (state[1] + offsets[blockIdx.x] + rank) % b.C : -1;
     __syncthreads();
-    // copy: warp w handles rows w, w + 8, ... of the block
-    for (int i = warp; i < RP_ROWS; i += RP_ROWS / 32) {
+    // copy: warp w handles rows w, w + THREADS / 32, ... of the block
+    for (int i = warp; i < ROWS; i += THREADS / 32) {
         const int64_t slot = slot_s[i];
         if (slot < 0) continue;
         const int64_t row = r0 + i;
@@ -299,15 +297,28 @@ int replay_push(fr_replay *rb, const fr_env *env, const fr_traj *tr, int32_t T, 
     cudaStream_t s = (cudaStream_t)stream;
     const int N = env->v.N;
     const int64_t rows = (int64_t)T * N;
-    const int64_t nb = (rows + RP_ROWS - 1) / RP_ROWS;
+    // Rows per block: 32 (two per warp) while that leaves the GPU with few rows in
+    // flight, so that a small push is as short as a row's copy: 256 rows of 301
+    // floats 9 us, 45 us in one block of 256, which copy 32 rows one after another
+    // per warp (65,536 rows 64 and 82 us); blocks of 256 rows beyond, whose fewer
+    // counts and threads cost less: 131,072 rows 115 us (119 in blocks of 32),
+    // 524,288 rows of 10 floats 161 us (220).
+    const int rpb = rows <= 65536 ? 32 : 256;
+    const int64_t nb = (rows + rpb - 1) / rpb;
     FR_CHECK(nb <= 0x7fffffffLL, FR_EINVAL, "replay_push: trajectory too large");
     int64_t *counts = nullptr;
     FR_CUDA(cudaMallocAsync((void **)&counts, (size_t)nb * 8, s));
     const int ar = env->v.auto_reset;
-    k_rp_count<<<(unsigned)nb, RP_ROWS, 0, s>>>(rows, N, tr->done, live0, ar, counts);
-    k_rp_scan<<<1, 1024, 0, s>>>(counts, (int)nb, rb->state);
-    k_rp_scatter<<<(unsigned)nb, RP_ROWS, 0, s>>>(rb->b, rows, N, ld, tr->obs, tr->act, tr->rew_f32, tr->done,
-                                                  last_obs, live0, ar, counts, rb->state);
+    auto push = [&](auto count, auto scatter, int threads) {
+        count<<<(unsigned)nb, rpb, 0, s>>>(rows, N, tr->done, live0, ar, counts);
+        k_rp_scan<<<1, 1024, 0, s>>>(counts, (int)nb, rb->state);
+        scatter<<<(unsigned)nb, threads, 0, s>>>(rb->b, rows, N, ld, tr->obs, tr->act, tr->rew_f32, tr->done,
+                                                    last_obs, live0, ar, counts, rb->state);
+    };
+    if (rpb == 32)
+        push(k_rp_count<32>, k_rp_scatter<32, 512>, 512);
+    else
+        push(k_rp_count<256>, k_rp_scatter<256, 256>, 256);
     const cudaError_t e = cudaGetLastError();
     cudaFreeAsync(counts, s);
     FR_CUDA(e);
