@@ -151,17 +151,19 @@ __device__ __forceinline__ TcUnit tc_unit(const TcPlan &p, const TcLayer &ly, in
 }
 
 // A warp's 32 observation rows from g0 in chunks of CK columns: put(v, rr, c)
-// gets chunk c of row rr (zeros past n rows and fin columns).  Lanes take 4
+// gets chunk c of row rr (zeros past fin columns; groups of rows past n are left
+// out: what an MMA makes of their operand rows is not stored).  Lanes take 4
 // rows x 8 chunks (16 rows x 2 where a row has fewer), and NB such groups'
 // loads are in flight: one row at a time, a pass over 32 rows was 32 load
-// latencies (65,536 rows x 5 agents of 10-128-128-3, BF16X3: Q targets 430 us, 316 now).
+// latencies (19,000 rows x 5 agents of 10-128-128-3, BF16X3: 68.9 -> 45.2 us;
+// one row of 3 x 320-256-256-30, BF16: 34.5 -> 27.2, with every group packed 31).
 template <int CK, int NB, class Put>
 __device__ __forceinline__ void obs_rows(const float *__restrict__ obs, int ld, int g0, int n, int fin, int chunks,
                                          int lane, Put put)
 {
     const int cl = chunks >= 8 ? 8 : 2, rl = 32 / cl;
     const int rr0 = lane % rl, c_lane = lane / rl;
-    for (int r0 = 0; r0 < 32; r0 += rl) {
+    for (int r0 = 0; r0 < 32 && g0 + r0 < n; r0 += rl) {
         const int rr = r0 + rr0, g = g0 + rr;
         const float *row = obs + (int64_t)g * ld;
         for (int c0 = c_lane; c0 < chunks; c0 += NB * cl) {
@@ -345,7 +347,6 @@ __global__ void __launch_bounds__(TC_THREADS) k_tc_forward(TcPlan plan, const ui
         fence_proxy_async_smem();
         mbar_arrive(a_ready);
         const uint32_t row_off = (uint32_t)(r / 8) * 128u + (uint32_t)(r % 8) * 16u;
-        uint32_t vn[16];                        // the second half of a pair of loads
         for (int l = 0; l < plan.L; ++l) {
             const TcLayer &ly = plan.layer[l];
             const bool last = l == plan.L - 1;
@@ -354,32 +355,18 @@ __global__ void __launch_bounds__(TC_THREADS) k_tc_forward(TcPlan plan, const ui
             const float *bl = bias + ((size_t)agent * MAX_LAYERS + l) * 256;
             const float *dl = dq + ((size_t)agent * MAX_LAYERS + l) * 256;          // FP8 only
             for (int c0 = 0; c0 < ly.N; c0 += 16) {
-                // two loads in flight per wait; bias and factors four columns per load
                 uint32_t v[16];
-                if ((c0 & 16) == 0) {
-                    __syncwarp();
-                    tmem_ld16(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)c0, v);
-                    if (c0 + 16 < ly.N) tmem_ld16(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)c0 + 16u, vn);
-                    tmem_ld_wait();
+                __syncwarp();
+                tmem_ld16(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)c0, v);
+                tmem_ld_wait();
+                float x[16];
+                if (fp8) {
+#pragma unroll
+                    for (int i = 0; i < 16; ++i)
+                        x[i] = __fmaf_rn(__uint_as_float(v[i]), __ldg(dl + c0 + i), __ldg(bl + c0 + i));
                 } else {
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) v[i] = vn[i];
-                }
-                float x[16];
-#pragma unroll
-                for (int i4 = 0; i4 < 4; ++i4) {
-                    const float4 b4 = __ldg((const float4 *)(bl + c0) + i4);
-                    const float bb[4] = {b4.x, b4.y, b4.z, b4.w};
-                    float dd[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-                    if (fp8) {
-                        const float4 d4 = __ldg((const float4 *)(dl + c0) + i4);
-                        dd[0] = d4.x; dd[1] = d4.y; dd[2] = d4.z; dd[3] = d4.w;
-                    }
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const float acc = __uint_as_float(v[4 * i4 + i]);
-                        x[4 * i4 + i] = fp8 ? __fmaf_rn(acc, dd[i], bb[i]) : acc + bb[i];
-                    }
+                    for (int i = 0; i < 16; ++i) x[i] = __uint_as_float(v[i]) + __ldg(bl + c0 + i);
                 }
                 if (!last && fp8) {
 #pragma unroll
