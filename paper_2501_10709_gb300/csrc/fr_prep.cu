@@ -15,9 +15,9 @@
 // 32 assets, one lane per asset) runs two chains, one warp each -- the SM takes
 // one FP64 instruction per 19 cycles, so two chains run at full rate and four
 // would not -- while a warp beside each prepares its inputs on the integer
-// pipe, 64 days ahead; every block takes an SM to itself (shared memory), so
-// nothing else competes for the pipe.  Window blocks in
-// the same launch (two assets x 128 days, one thread per day) stage the tile
+// pipe, 64 days ahead; where the chains set the time every block takes an SM to
+// itself (shared memory), so nothing else competes for the pipe.  Window blocks
+// in the same launch (two assets x 128 days, one thread per day) stage the tile
 // plus a 59-day halo of closes and typical prices in shared memory and compute
 // the windowed means, the standard deviation and the mean absolute deviation.
 // A second launch, one thread per (day, asset), turns the chains' states into
@@ -39,9 +39,10 @@ constexpr int N_IND = 8;
 constexpr int PREP_SEG = 64;       // days a chain's inputs are prepared ahead
 constexpr int PREP_THREADS = 256;
 constexpr int N_PLANES = 7;        // chain states: gains, losses, TR, DM+, DM-, EMA-12, EMA-26
-constexpr size_t PREP_SMEM = 128 * 1024;   // one block per SM
 constexpr int CHAINS = 2;          // chains per block
-static_assert(PREP_SMEM >= sizeof(double) * CHAINS * 2 * PREP_SEG * 32, "input buffers of a chain block");
+constexpr size_t PREP_SMEM = sizeof(double) * CHAINS * 2 * PREP_SEG * 32;   // input buffers of a chain block: 64 KB
+constexpr size_t PREP_ALONE = 128 * 1024;  // one block per SM
+static_assert(PREP_SMEM >= sizeof(double) * 4 * (PREP_TILE + PREP_HALO), "window blocks' tiles");
 
 __device__ __forceinline__ double dadd(double a, double b) { return __dadd_rn(a, b); }
 __device__ __forceinline__ double dsub(double a, double b) { return __dsub_rn(a, b); }
@@ -342,14 +343,20 @@ cudaError_t launch_indicators(const int64_t *close, const int64_t *high, const i
     const int n_chain = 4 * ((K + 31) / 32), n_tiles = (T + PREP_TILE - 1) / PREP_TILE;
     const long long blocks = (long long)n_chain + (long long)((K + 1) / 2) * n_tiles;
     if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
-    int dev = 0;
+    int dev = 0, sms = 1;
     cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    // Blocks share SMs (three each) where they are more than the chains' length
+    // pays for alone, about 75 days a wave: 60 days x 3,000 assets 214 us shared, 256
+    // alone, 1,000 x 600 604 and 642; 1,000 x 300 368 and 335, 2,520 x 100 535 and
+    // 419.
+    const size_t smem = blocks > sms && blocks * 75 > (long long)sms * T ? PREP_SMEM : PREP_ALONE;
     if (e == cudaSuccess) e = set_max_smem_once((const void *)k_indicators, dev);
     // the chains' states, stream-ordered scratch: 7 doubles per (day, asset)
     double *st = nullptr;
     if (e == cudaSuccess) e = cudaMallocAsync((void **)&st, 8ull * N_PLANES * (uint64_t)T * K, s);
     if (e != cudaSuccess) return e;
-    k_indicators<<<(unsigned)blocks, PREP_THREADS, PREP_SMEM, s>>>(close, high, low, T, K, ind, n_chain, n_tiles, st);
+    k_indicators<<<(unsigned)blocks, PREP_THREADS, smem, s>>>(close, high, low, T, K, ind, n_chain, n_tiles, st);
     e = cudaGetLastError();
     if (e == cudaSuccess) {
         k_ind_final<<<ceil_div((int64_t)T * K, 256), 256, 0, s>>>(close, T, K, st, ind);
