@@ -195,7 +195,7 @@ __device__ __forceinline__ void wd_combine(const WdArgs &a, WdBars *bars, uint8_
     const int fout = p.layer[2].fout, lane = threadIdx.x & 31;
     volatile int *abort = &bars->abort;
     const uint32_t comb = smem_u32(base + a.comb);
-    const float *w = bars->w[(threadIdx.x >> 5) & 3];
+    const uint32_t w = smem_u32(bars->w[(threadIdx.x >> 5) & 3]);
     uint32_t far = 0u, far_bar = 0u;
     if (agent > 0) {
         far = map_shared_rank(comb, (uint32_t)c) + (uint32_t)(((agent - 1) * n + r) * 128);
@@ -222,9 +222,10 @@ __device__ __forceinline__ void wd_combine(const WdArgs &a, WdBars *bars, uint8_
             for (int j = 1; j < p.M; ++j) {
                 const uint4 o = ld_shared_v4(comb + (uint32_t)(((j - 1) * n + r) * 128 + k0 * 4));
                 const uint32_t ou[4] = {o.x, o.y, o.z, o.w};
+                const float wj = ld_shared_f32(w + 4u * (uint32_t)j);
 #pragma unroll
                 for (int u = 0; u < 4; ++u)
-                    acc[u] = __fadd_rn(acc[u], __fmul_rn(w[j], __fsub_rn(__uint_as_float(ou[u]), x[u])));
+                    acc[u] = __fadd_rn(acc[u], __fmul_rn(wj, __fsub_rn(__uint_as_float(ou[u]), x[u])));
             }
 #pragma unroll
             for (int u = 0; u < 4; ++u)
@@ -607,8 +608,12 @@ int wd_most(const TcPlan &p, bool act, int optin)
 // nothing else that does may share their SMs (two clusters, each holding one
 // SM's tensor memory and waiting for the other's, would wait for ever; beside
 // the 64-row kernel's registers a CTA of the first fused crypto kernel fits):
-// they take the whole shared memory too.
-uint32_t wd_smem(uint32_t layout, int size, int optin) { return size > 1 ? (uint32_t)optin : layout + 1024u; }
+// they take the shared memory too, but for 8 KB, where the combining kernel's
+// blocks fit and no such CTA (14 KB at least for its 32 columns).
+uint32_t wd_smem(uint32_t layout, int size, int optin)
+{
+    return size > 1 ? std::max(layout + 1024u, (uint32_t)optin - 8192u) : layout + 1024u;
+}
 
 // Clusters of `size` CTAs the device holds at once (each CTA has an SM to
 // itself), queried once per device, size and shared memory; 0 when it holds
