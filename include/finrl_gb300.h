@@ -362,8 +362,9 @@ int ensemble_act(const fr_ensemble *ens, const float *obs, int32_t n,
  * that owns every device buffer and forbids a library from allocating behind
  * its back.  The paper has no counterpart; this is a library convenience.
  * Same arguments, layouts and results as ensemble_act (on the tensor-core
- * precisions it always runs the single-agent kernel, which gives the same
- * results as the large-batch one).  Its scratch is a fixed 16 MiB array
+ * precisions it never runs the large-batch kernel, whose results are the same
+ * but for a NaN in a hidden layer: it stays NaN there, in batches of at least one
+ * 128-row tile per SM, and becomes 0 elsewhere).  Its scratch is a fixed 16 MiB array
  * inside the library image (held on every GPU that loads the library until
  * the process exits), so no cudaMalloc, cudaFree or other allocating routine
  * is called.  A batch whose scratch would not fit (roughly
@@ -515,13 +516,15 @@ int env_set_table_cache(fr_env *env, int32_t on);
 /* Split fused rollouts (no counterpart in the paper).  on = 1 (the default):
  * a fused stock rollout, or a BF16 / FP16 crypto rollout whose tiles leave
  * SMs idle, of T >= 128 steps, without tile packing, trajectory outputs or
- * auto-reset, runs as K = min(4, T / 64) launches of the resident kernel (the last T / 8 steps, the one before it T / 4, the
- * others sharing the rest evenly) on an internal stream of the highest
- * priority, and the FP64 metrics replay of each piece runs on `stream`
+ * auto-reset, runs as K = min(4, T / 64) launches of the resident kernel (the
+ * last T / 8 steps, the one before it T / 4, the others sharing the rest
+ * evenly) on an internal stream of the highest priority, and the FP64 metrics replay of each piece runs on `stream`
  * beside the next piece, so that only the last piece's replay follows the
  * kernel.  Events order the two streams, so the rollout is still one
  * ordered operation on `stream` and can be captured into a graph.  Results
- * are those of one launch, bit for bit.  on = 0: always one launch. */
+ * are those of one launch, bit for bit.  A crypto rollout is one launch too
+ * where the budget, or in a capture the env's scratch, has room for its value
+ * log alone.  on = 0: always one launch. */
 int env_set_rollout_split(fr_env *env, int32_t on);
 
 /* Autotuner of the batched rollouts (no counterpart in the paper: the

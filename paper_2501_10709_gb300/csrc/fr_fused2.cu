@@ -207,8 +207,6 @@ __host__ __device__ inline F2Smem f2_smem(const F2Plan &p)
     return s;
 }
 
-// pieces of a split rollout (launches of the resident kernel per rollout)
-
 // barrier slots
 enum { B_W = 0, B_OBS, B_ACC, B_H1, B_H2, B_X, B_END, B_COUNT };
 

@@ -1,7 +1,9 @@
-// fr_plain.cu -- the plain, unfused FP32 actor path: one SIMT dense-layer
-// kernel launch per layer (all agents of the ensemble in one grid), then a
-// separate combine launch.  It is the comparison path for the fused BF16
-// rollout and the fp32 reference the tensor-core kernels are held to.
+// fr_plain.cu -- the plain, unfused FP32 actor path: the whole network in one
+// SIMT launch (k_mlp_f32: layer inputs up to 304 wide, outputs up to 256), or a
+// dense-layer launch per layer (k_dense_f32: wider inputs), all agents of the
+// ensemble in one grid; then a separate combine launch.  It is the comparison
+// path for the fused BF16 rollout and the fp32 reference the tensor-core kernels
+// are held to.
 #include "fr_common.cuh"
 #include "fr_ptx.cuh"
 
