@@ -397,9 +397,9 @@ int nw_rollout(fr_env *env, const fr_ensemble *e, int T, const fr_traj *traj, vo
 bool tc_rollout_supported(const fr_env *env, const fr_ensemble *e);
 // FP64 episode accumulators from a rollout's value log (fr_fused.cu)
 // t0 (NULL: the env's step counters) gives each env's step count before the
-// logged steps.  With t0 the caller has already advanced the counters: the
-// replay without auto-reset leaves them alone, the one with auto-reset
-// writes them (its count restarts with every episode, as the kernel's).
+// logged steps.  With t0 the kernel that logged them has advanced the counters,
+// and the next piece of the rollout may do so again beside the replay, which
+// leaves them alone.
 cudaError_t launch_metrics_replay(const EnvView &v, const int64_t *vlog, int T, double *metrics,
                                   cudaStream_t s, const int32_t *t0 = nullptr);
 // whether one thread per env is the faster form (fr_metrics.cu) for the replay of

@@ -832,7 +832,7 @@ __global__ void __launch_bounds__(FU_THREADS, TASK == FR_TASK_CRYPTO ? 3 : 1)
 }
 
 // Replays the value log through the FP64 episode accumulators in time order
-// (one thread per env), advancing the step counters, latching finished
+// (one thread per env), advancing the step counters (without t0), latching finished
 // episodes under auto-reset, and writing the metrics when asked.
 __global__ void k_metrics_replay(EnvView v, const int64_t *vlog, int T, double *metrics, const int32_t *t0)
 {
@@ -863,7 +863,9 @@ __global__ void k_metrics_replay(EnvView v, const int64_t *vlog, int T, double *
     v.mdd[e] = mdd;
     v.peak[e] = peak;
     v.vlast[e] = vlast;
-    v.t[e] = n;
+    // with t0 the kernel that wrote the log advances the count, and the next
+    // piece of the rollout may have done so again
+    if (!t0) v.t[e] = n;
     if (metrics) {
         double *o = metrics + (int64_t)e * 3;
         if (n == 0 && Lt[3] != 0.0) {

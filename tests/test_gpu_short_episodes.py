@@ -53,3 +53,27 @@ def test_replay_of_a_short_log_equals_stepping(ctx, dev, N, pieces):
         fr.env_metrics(b, mb)
         torch.cuda.synchronize()
         assert torch.equal(ma, mb)
+
+
+def test_rollout_of_many_envs_in_pieces(ctx, dev):
+    # the pieces' replays, one thread per env at this many envs, run beside the
+    # next pieces, which take the step counts from the kernel alone
+    N, T = 20_000, 256
+    mk = fr.fr_market_create(ctx, synth.stock_market(700, 30, seed=3))
+    e = synth.stock_envs_cohorts(N, 30, 700, 2 * T, 8, 3)
+    dims = (301, 64, 64, 30)
+    ens = fr.ensemble_create(ctx, dims, synth.actor_params(dims, 3, seed=3), precision=fr.PREC_BF16)
+    out = []
+    for split in (False, True):
+        env = fr.env_create(ctx, mk, start=e.start, window=e.W, n_assets=e.Ke, bps=e.bps)
+        fr.env_set_rollout_split(env, split)
+        got = []
+        for steps in (T, 130):
+            m = torch.empty(N, 3, dtype=torch.float64, device=dev)
+            fr.rollout(env, ens, steps, metrics=m)
+            st = [torch.empty(N, dtype=t, device=dev) for t in (torch.int64, torch.int32, torch.uint8)]
+            fr.env_get_state(env, cash=st[0], steps=st[1], done=st[2])
+            got += [m] + st
+        torch.cuda.synchronize()
+        out.append(got)
+    assert all(torch.equal(x, y) for x, y in zip(*out))
