@@ -79,6 +79,7 @@ struct WdArgs {
     int act;                                      // 1: y is the weighted mean of the agents [rows][outputs]
     const float *w;                               // the agents' weights (device), read by every launch and replay
     uint32_t x_bytes, h_bytes, stage_bytes, w3, x, h1, h2, stage, comb, bars;   // shared memory
+    uint32_t cw;                                  // after comb: the weights, a copy per output warp
     int bulk;                                     // rows are packed and 16-byte aligned: bulk copies
 };
 
@@ -93,7 +94,6 @@ struct WdBars {
     uint64_t drain;
     uint32_t tmem;
     int abort;
-    float w[4][MAX_AGENTS];                       // combine weights, a copy per output warp
 };
 
 __device__ __forceinline__ void wd_wait(uint64_t *bar, uint32_t parity, bool remote, volatile int *abort,
@@ -195,7 +195,7 @@ __device__ __forceinline__ void wd_combine(const WdArgs &a, WdBars *bars, uint8_
     const int fout = p.layer[2].fout, lane = threadIdx.x & 31;
     volatile int *abort = &bars->abort;
     const uint32_t comb = smem_u32(base + a.comb);
-    const uint32_t w = smem_u32(bars->w[(threadIdx.x >> 5) & 3]);
+    const uint32_t w = smem_u32(base + a.cw) + ((threadIdx.x >> 5) & 3u) * (uint32_t)(4 * MAX_AGENTS);
     uint32_t far = 0u, far_bar = 0u;
     if (agent > 0) {
         far = map_shared_rank(comb, (uint32_t)c) + (uint32_t)(((agent - 1) * n + r) * 128);
@@ -393,7 +393,7 @@ __global__ void __launch_bounds__(WD_THREADS, 1) k_wide(const __grid_constant__ 
         const float bl = lane < l3.N ? b3[lane] : 0.0f;
         grid_wait_previous();                              // whatever still reads the outputs
         if (a.act) {
-            if (lane < p.M) bars->w[q][lane] = a.w[lane];
+            if (lane < p.M) ((float *)(base + a.cw))[q * MAX_AGENTS + lane] = a.w[lane];
             __syncwarp();
         }
         for (int m = 0; m < owned; ++m) {
@@ -587,6 +587,7 @@ uint32_t wd_layout(const TcPlan &p, WdArgs *a)
     a->w3 = take((uint32_t)(WD_OUTS * p.layer[2].K) * 2u);
     a->stage = take(WD_LOADERS * a->stage_bytes);
     a->comb = a->act ? take((uint32_t)((p.M - 1) * a->n * WD_OUTS * 4)) : 0u;
+    a->cw = a->act ? take(4u * MAX_AGENTS * sizeof(float)) : 0u;
     a->bars = take(sizeof(WdBars));
     return off;
 }
