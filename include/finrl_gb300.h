@@ -518,9 +518,9 @@ int env_set_table_cache(fr_env *env, int32_t on);
  * SMs idle, of T >= 128 steps, without tile packing, trajectory outputs or
  * auto-reset, runs as K = min(4, T / 64) launches of the resident kernel (the
  * last T / 8 steps, the one before it T / 4, the others sharing the rest
- * evenly) on an internal stream of the highest priority, and the FP64 metrics replay of each piece runs on `stream`
- * beside the next piece, so that only the last piece's replay follows the
- * kernel.  Events order the two streams, so the rollout is still one
+ * evenly) on an internal stream of the highest priority, and the FP64 metrics
+ * replay of each piece runs on `stream` beside the next piece, so that only the
+ * last piece's replay follows the kernel.  Events order the two streams, so the rollout is still one
  * ordered operation on `stream` and can be captured into a graph.  Results
  * are those of one launch, bit for bit.  A crypto rollout is one launch too
  * where the budget, or in a capture the env's scratch, has room for its value
