@@ -156,7 +156,7 @@ __device__ __forceinline__ TcUnit tc_unit(const TcPlan &p, const TcLayer &ly, in
 // rows x 8 chunks (16 rows x 2 where a row has fewer), and NB such groups'
 // loads are in flight: one row at a time, a pass over 32 rows was 32 load
 // latencies (19,000 rows x 5 agents of 10-128-128-3, BF16X3: 68.9 -> 45.2 us;
-// one row of 3 x 320-256-256-30, BF16: 34.5 -> 27.2, with every group packed 31).
+// one row of 3 x 320-256-256-30, BF16: 34.5 -> 27.2).
 template <int CK, int NB, class Put>
 __device__ __forceinline__ void obs_rows(const float *__restrict__ obs, int ld, int g0, int n, int fin, int chunks,
                                          int lane, Put put)

@@ -720,7 +720,7 @@ bool wd_ok(const fr_ensemble *e)
 // (26 us per agent over CTA pairs, 15.5 in single CTAs, 4 for more than 16
 // outputs, and the loading), while the tiled kernel, which converts the rows
 // once for every agent, pays for the columns that there are and for whole waves.
-// Fitted to 560 shapes at 19,455 .. 262,144 rows; what it picks is at most 5%
+// Fitted to 459 shapes at 19,455 .. 262,144 rows; what it picks is at most 5%
 // behind the better one (3 x 10-144-96-3 on 262,144 rows: 212 us tiled, 258
 // here; 8 x 304-16-256-30 on 77,824: 267 and 410; 3 x 301-256-256-30: 164 and
 // 127).
@@ -755,7 +755,7 @@ int wd_prepare(const fr_ensemble *e)
     // Combining in the same launch: a cluster holds every agent (at most eight
     // CTAs), 48 rows a tile.  It spares small batches, which wait for the host,
     // an allocation and a launch (8 rows of 3 x 301-256-256-30: 12.3 us a call),
-    // but the GPU holds few such clusters (23 of six, 14 of eight), so that past
+    // but the GPU holds few such clusters (23 of six, 15 of eight), so that past
     // two waves of them a forward over every SM and a combining launch are faster
     // on the GPU by more than they cost the host: 8 x 61-64-64-30 on 4,096 rows
     // 54 us combined, 20 us in two launches; 3 x 301-256-256-30 on 3,072 rows 24
